@@ -1276,7 +1276,7 @@ int dda_scattering_cross_section(dda_ctx* c, const void* p, double* out, void* s
     if (int rc = launch_matvec<double>(m, P, c->aux[2], st)) return rc;        // A^H P
     if (int rc = launch_csca(target_view(c), c->g, c->k, c->ainv64, P, c->aux[1], c->aux[2], c->xsec, st)) return rc;
     double2 h;
-    DDA_CUDA_TRY(cudaMemcpyAsync(&h, c->xsec + xsec_scratch_elems() - 1, sizeof(double2), cudaMemcpyDeviceToHost, st));
+    DDA_CUDA_TRY(cudaMemcpyAsync(&h, c->xsec, sizeof(double2), cudaMemcpyDeviceToHost, st));
     DDA_CUDA_TRY(cudaStreamSynchronize(st));
     *out = 4.0 * M_PI * c->k * h.x;
     return DDA_OK;
@@ -1330,21 +1330,23 @@ int dda_cross_sections_batch(dda_ctx* c, int nb, const void* einc, const void* p
         DDA_CUDA_TRY(cudaMemcpyAsync(c->sp.r64, p, bytes, cudaMemcpyHostToDevice, st));
         P = c->sp.r64;
     }
-    // one reduction per right-hand side; each result is copied out before
-    // the next one reuses the scratch (stream order)
-    double2* h = reinterpret_cast<double2*>(c->sp.host);   // pinned, >= nb double2
-    for (int b = 0; b < nb; ++b) {
-        if (int rc = launch_cross_sections(target_view(c), c->g, c->k, c->ainv64, E + b * n, P + b * n, c->xsec, st))
-            return rc;
-        DDA_CUDA_TRY(cudaMemcpyAsync(h + b, c->xsec + xsec_scratch_elems() - 1, sizeof(double2),
-                                     cudaMemcpyDeviceToHost, st));
-    }
-    DDA_CUDA_TRY(cudaStreamSynchronize(st));
+    // kXsecBatch right-hand sides per launch; their sums come back through
+    // the pinned state (at least one KState)
+    static_assert(sizeof(KState) >= kXsecBatch * sizeof(double2), "pinned buffer of the cross sections");
+    const double2* h = reinterpret_cast<const double2*>(c->sp.host);
     const double f = 4.0 * M_PI * c->k;
-    for (int b = 0; b < nb; ++b) {
-        out[3 * b] = f * h[b].x;
-        out[3 * b + 1] = f * h[b].y;
-        out[3 * b + 2] = out[3 * b] - out[3 * b + 1];
+    for (int b0 = 0; b0 < nb; b0 += kXsecBatch) {
+        const int m = std::min(kXsecBatch, nb - b0);
+        if (int rc = launch_cross_sections(target_view(c), c->g, c->k, c->ainv64, m, E + b0 * n, P + b0 * n, c->xsec, st))
+            return rc;
+        DDA_CUDA_TRY(cudaMemcpyAsync(c->sp.host, c->xsec, m * sizeof(double2), cudaMemcpyDeviceToHost, st));
+        DDA_CUDA_TRY(cudaStreamSynchronize(st));
+        for (int b = 0; b < m; ++b) {
+            double* o = out + 3 * (b0 + b);
+            o[0] = f * h[b].x;
+            o[1] = f * h[b].y;
+            o[2] = o[0] - o[1];
+        }
     }
     return DDA_OK;
 }

@@ -2,6 +2,7 @@
 // set-up and observables on it: occupancy / composition packing, the rank
 // (compressed index) of every site for the zero-storage vectors of Sec. 4,
 // the incident field and the cross-section sums.
+#include <cmath>
 #include <mutex>
 
 #include "target.cuh"
@@ -147,77 +148,167 @@ __global__ void k_site_ranks(TargetView tv, int64_t n, uint32_t* __restrict__ ou
 }
 
 // --------------------------------------------------------- incident field
-__global__ void k_incident(TargetView tv, Geometry g, double kw, double kx, double ky, double kz, double2 e0,
-                           double2 e1, double2 e2, double2* __restrict__ E) {
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < g.nsites; s += stride) {
-        if (!occupied(tv, s)) continue;
-        const int i = (int)(s % g.K), j = (int)((s / g.K) % g.J), k = (int)(s / ((int64_t)g.K * g.J));
-        double sn, cs;
-        sincos(kw * (kx * i + ky * j + kz * k), &sn, &cs);
-        const double2 ph = make_double2(cs, sn);
-        const uint32_t r = site_rank(tv, s);
-        E[r] = cmul<double>(e0, ph);
-        E[g.nd + r] = cmul<double>(e1, ph);
-        E[2 * g.nd + r] = cmul<double>(e2, ph);
+// E = e exp(i k khat . r) = [e exp(i k (khat_y j + khat_z k))] exp(i k khat_x i):
+// one phase per row (j, k) and one per x index, so that a site costs three
+// complex products instead of a sine and cosine (FP64 arithmetic bounds this
+// kernel: at 200^3, 4.19 M sites, it took 424 us with a sincos per site,
+// 126 us this way; writing the field alone takes 30 us at the measured copy
+// rate).  A CTA takes the rows b, b + G, ...
+// (interleaved: a target's first and last planes are often nearly empty),
+// kIncRows at a time.
+constexpr int kIncThreads = 512;
+constexpr int kIncRows = 128;
+constexpr int kIncUnroll = 4;
+
+// one axis of the wave vector as an unevaluated sum of two doubles, and the
+// phase n of that axis added to an angle held the same way
+struct Angle { double hi, lo; };
+__device__ __forceinline__ Angle angle_at(Angle a, int n) {
+    const double p = a.hi * n;
+    return Angle{p, fma(a.hi, (double)n, -p) + a.lo * n};
+}
+__device__ __forceinline__ Angle angle_add(Angle a, Angle b) {
+    const double s = a.hi + b.hi, v = s - a.hi;
+    return Angle{s, (a.hi - (s - v)) + (b.hi - v) + a.lo + b.lo};
+}
+__device__ __forceinline__ double2 phase(Angle a) {
+    double sn, cs;
+    sincos(a.hi, &sn, &cs);
+    return make_double2(cs - sn * a.lo, sn + cs * a.lo);   // |lo| is a rounding error of hi
+}
+
+__global__ void __launch_bounds__(kIncThreads) k_incident(TargetView tv, Geometry g, Angle ax, Angle ay, Angle az,
+                                                          double2 e0, double2 e1, double2 e2,
+                                                          double2* __restrict__ E) {
+    __shared__ double2 px[kMaxEdge];
+    __shared__ double2 F[kIncRows][3];
+    const int nrows = g.J * g.P, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int i = threadIdx.x; i < g.K; i += kIncThreads) px[i] = phase(angle_at(ax, i));
+    for (int base = blockIdx.x; base < nrows; base += kIncRows * gridDim.x) {
+        const int left = (nrows - base + gridDim.x - 1) / gridDim.x, cnt = left < kIncRows ? left : kIncRows;
+        __syncthreads();
+        if (threadIdx.x < cnt) {
+            const int row = base + threadIdx.x * gridDim.x;
+            const double2 f = phase(angle_add(angle_at(ay, row % g.J), angle_at(az, row / g.J)));
+            F[threadIdx.x][0] = cmul<double>(e0, f);
+            F[threadIdx.x][1] = cmul<double>(e1, f);
+            F[threadIdx.x][2] = cmul<double>(e2, f);
+        }
+        __syncthreads();
+        for (int q = warp; q < cnt; q += kIncThreads / 32) {
+            const int s0 = (base + q * gridDim.x) * g.K;
+            for (int i0 = lane; i0 < g.K; i0 += 32 * kIncUnroll) {
+                uint32_t word[kIncUnroll], rank[kIncUnroll];
+#pragma unroll
+                for (int u = 0; u < kIncUnroll; ++u) {
+                    const int i = i0 + 32 * u;
+                    word[u] = i < g.K ? __ldg(tv.occ + ((s0 + i) >> 5)) : 0u;
+                    rank[u] = i < g.K ? __ldg(tv.rank + ((s0 + i) >> 5)) : 0u;
+                }
+#pragma unroll
+                for (int u = 0; u < kIncUnroll; ++u) {
+                    const int i = i0 + 32 * u, bit = (s0 + i) & 31;
+                    if (!((word[u] >> bit) & 1u)) continue;
+                    const int64_t r = rank[u] + __popc(word[u] & ((1u << bit) - 1u));
+                    const double2 x = px[i];
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) E[c * g.nd + r] = cmul<double>(F[q][c], x);
+                }
+            }
+        }
     }
 }
 
 // --------------------------------------------------------- cross sections
-// per block partial sums of Im(E^* P) and [-Im(ainv) - 2/3 k^3] |P|^2 over
-// sites; the final sum over blocks runs in a fixed order on one block
+// per block partial sums of Im(E^* P) and [-Im(ainv) - 2/3 k^3] |P|^2; the
+// final sum over blocks runs in a fixed order on one block per right-hand
+// side.  FP64 arithmetic and HBM bound it about equally: with one material
+// the weight is a constant of the component, so the compressed vectors are
+// streamed without a look at the bit field and a value costs four FP64
+// operations; with more, each occupied site looks its materials up and takes
+// the weights from shared memory.
 constexpr int kRedThreads = 256;
 constexpr int kRedBlocks = 1024;
+constexpr int kRedUnroll = 4;
 
+// sums of a and b over the block, valid in thread 0
+__device__ __forceinline__ double2 block_sum2(double a, double b) {
+    __shared__ double sa[kRedThreads / 32], sb[kRedThreads / 32];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        a += __shfl_down_sync(0xffffffffu, a, o);
+        b += __shfl_down_sync(0xffffffffu, b, o);
+    }
+    if ((threadIdx.x & 31) == 0) { sa[threadIdx.x >> 5] = a; sb[threadIdx.x >> 5] = b; }
+    __syncthreads();
+    double2 t = make_double2(0.0, 0.0);
+    if (threadIdx.x == 0)
+        for (int w = 0; w < kRedThreads / 32; ++w) { t.x += sa[w]; t.y += sb[w]; }
+    return t;
+}
+
+// grid (blocks per right-hand side, right-hand sides)
+template <bool ONE>
 __global__ void __launch_bounds__(kRedThreads) k_xsec_partial(TargetView tv, Geometry g, double k3,
                                                               const double2* __restrict__ ainv,
                                                               const double2* __restrict__ E,
                                                               const double2* __restrict__ P,
                                                               double2* __restrict__ part) {
-    double ext = 0.0, abs_ = 0.0;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < g.nsites; s += stride) {
-        if (!occupied(tv, s)) continue;
-        const uint32_t r = site_rank(tv, s);
-        for (int c = 0; c < 3; ++c) {
-            const double2 e = E[c * g.nd + r], p = P[c * g.nd + r];
-            ext += e.x * p.y - e.y * p.x;                       // Im(conj(e) p)
-            const double2 a = ainv[material(tv, s, c) * 3 + c];
-            abs_ += (-a.y - (2.0 / 3.0) * k3) * (p.x * p.x + p.y * p.y);
-        }
-    }
-    __shared__ double se[kRedThreads], sa[kRedThreads];
-    se[threadIdx.x] = ext;
-    sa[threadIdx.x] = abs_;
+    extern __shared__ double weight[];   // [nmat][3]
+    for (int i = threadIdx.x; i < 3 * g.nmat; i += kRedThreads) weight[i] = -ainv[i].y - (2.0 / 3.0) * k3;
     __syncthreads();
-    for (int o = kRedThreads / 2; o > 0; o >>= 1) {
-        if (threadIdx.x < o) {
-            se[threadIdx.x] += se[threadIdx.x + o];
-            sa[threadIdx.x] += sa[threadIdx.x + o];
+    E += (int64_t)blockIdx.y * 3 * g.nd;
+    P += (int64_t)blockIdx.y * 3 * g.nd;
+    double ext = 0.0, abs_ = 0.0;
+    const int stride = gridDim.x * kRedThreads, first = blockIdx.x * kRedThreads + threadIdx.x;
+    if (ONE) {
+        const int nd = (int)g.nd;
+        for (int c = 0; c < 3; ++c) {
+            const double2 *Ec = E + c * g.nd, *Pc = P + c * g.nd;
+            double sq = 0.0;
+            for (int i = first; i < nd; i += kRedUnroll * stride) {
+                double2 e[kRedUnroll], p[kRedUnroll];
+#pragma unroll
+                for (int u = 0; u < kRedUnroll; ++u) {
+                    const int n = i + u * stride;
+                    e[u] = n < nd ? Ec[n] : make_double2(0.0, 0.0);
+                    p[u] = n < nd ? Pc[n] : make_double2(0.0, 0.0);
+                }
+#pragma unroll
+                for (int u = 0; u < kRedUnroll; ++u) {
+                    ext = fma(e[u].x, p[u].y, fma(-e[u].y, p[u].x, ext));   // Im(conj(e) p)
+                    sq = fma(p[u].x, p[u].x, fma(p[u].y, p[u].y, sq));
+                }
+            }
+            abs_ += weight[c] * sq;
         }
-        __syncthreads();
+    } else {
+        const int n = (int)g.nsites;
+        for (int s = first; s < n; s += stride) {
+            if (!occupied(tv, s)) continue;
+            const uint32_t r = site_rank(tv, s);
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                const double2 e = E[c * g.nd + r], p = P[c * g.nd + r];
+                ext = fma(e.x, p.y, fma(-e.y, p.x, ext));
+                abs_ = fma(weight[material(tv, s, c) * 3 + c], fma(p.x, p.x, p.y * p.y), abs_);
+            }
+        }
     }
-    if (threadIdx.x == 0) part[blockIdx.x] = make_double2(se[0], sa[0]);
+    const double2 t = block_sum2(ext, abs_);
+    if (threadIdx.x == 0) part[blockIdx.y * gridDim.x + blockIdx.x] = t;
 }
 
+// out[b] = sum of the n partials of right-hand side b = blockIdx.x
 __global__ void __launch_bounds__(kRedThreads) k_xsec_final(const double2* __restrict__ part, int n, double2* out) {
-    __shared__ double se[kRedThreads], sa[kRedThreads];
     double e = 0.0, a = 0.0;
     for (int i = threadIdx.x; i < n; i += kRedThreads) {
-        e += part[i].x;
-        a += part[i].y;
+        const double2 p = part[blockIdx.x * n + i];
+        e += p.x;
+        a += p.y;
     }
-    se[threadIdx.x] = e;
-    sa[threadIdx.x] = a;
-    __syncthreads();
-    for (int o = kRedThreads / 2; o > 0; o >>= 1) {
-        if (threadIdx.x < o) {
-            se[threadIdx.x] += se[threadIdx.x + o];
-            sa[threadIdx.x] += sa[threadIdx.x + o];
-        }
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) *out = make_double2(se[0], sa[0]);
+    const double2 t = block_sum2(e, a);
+    if (threadIdx.x == 0) out[blockIdx.x] = t;
 }
 
 // C_sca as the exact pair sum of the radiated power,
@@ -247,14 +338,8 @@ __global__ void __launch_bounds__(kRedThreads) k_csca_partial(TargetView tv, Geo
             acc += ((2.0 / 3.0) * k3 + a.y) * (p.x * p.x + p.y * p.y) - re;
         }
     }
-    __shared__ double sa[kRedThreads];
-    sa[threadIdx.x] = acc;
-    __syncthreads();
-    for (int o = kRedThreads / 2; o > 0; o >>= 1) {
-        if (threadIdx.x < o) sa[threadIdx.x] += sa[threadIdx.x + o];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) part[blockIdx.x] = make_double2(sa[0], 0.0);
+    const double2 t = block_sum2(acc, 0.0);
+    if (threadIdx.x == 0) part[blockIdx.x] = t;
 }
 
 // right-hand side of the adjoint solve A mu = b (A complex symmetric):
@@ -389,21 +474,34 @@ int launch_site_ranks(const TargetView& tv, int64_t n, uint32_t* out, cudaStream
 
 int launch_incident(const TargetView& tv, const Geometry& g, double k, const double* khat, const double* e0,
                     double2* E, cudaStream_t st) {
-    k_incident<<<grid_for(g.nsites, 256), 256, 0, st>>>(tv, g, k, khat[0], khat[1], khat[2],
-                                                      make_double2(e0[0], e0[1]), make_double2(e0[2], e0[3]),
-                                                      make_double2(e0[4], e0[5]), E);
+    Angle a[3];
+    for (int i = 0; i < 3; ++i) {
+        a[i].hi = k * khat[i];
+        a[i].lo = std::fma(k, khat[i], -a[i].hi);
+    }
+    // at least a row per warp, at most two CTAs per SM (each one computes the K phases of the x axis)
+    const int rows = g.J * g.P, per = kIncThreads / 32;
+    const unsigned grid = (unsigned)std::min(152 * 2, (rows + per - 1) / per);
+    k_incident<<<grid, kIncThreads, 0, st>>>(tv, g, a[0], a[1], a[2], make_double2(e0[0], e0[1]),
+                                             make_double2(e0[2], e0[3]), make_double2(e0[4], e0[5]), E);
     DDA_LAUNCH_CHECK("incident field");
     return 0;
 }
 
-size_t xsec_scratch_elems() { return kRedBlocks + 1; }
+size_t xsec_scratch_elems() { return kRedBlocks + kXsecBatch; }
 
-int launch_cross_sections(const TargetView& tv, const Geometry& g, double k, const double2* ainv,
+int launch_cross_sections(const TargetView& tv, const Geometry& g, double k, const double2* ainv, int nb,
                           const double2* E, const double2* P, double2* scratch, cudaStream_t st) {
-    const unsigned blocks = (unsigned)std::min<int64_t>(kRedBlocks, std::max<int64_t>(1, (g.nsites + kRedThreads - 1) / kRedThreads));
-    k_xsec_partial<<<blocks, kRedThreads, 0, st>>>(tv, g, k * k * k, ainv, E, P, scratch);
+    const bool one = g.nmat == 1;
+    const int64_t need = ((one ? g.nd : g.nsites) + kRedThreads - 1) / kRedThreads;
+    const unsigned blocks = (unsigned)std::max<int64_t>(1, std::min<int64_t>(kRedBlocks / nb, need));
+    const size_t sm = 3 * (size_t)g.nmat * sizeof(double);
+    const dim3 grid(blocks, nb);
+    double2* part = scratch + kXsecBatch;
+    if (one) k_xsec_partial<true><<<grid, kRedThreads, sm, st>>>(tv, g, k * k * k, ainv, E, P, part);
+    else k_xsec_partial<false><<<grid, kRedThreads, sm, st>>>(tv, g, k * k * k, ainv, E, P, part);
     DDA_LAUNCH_CHECK("cross-section partial sums");
-    k_xsec_final<<<1, kRedThreads, 0, st>>>(scratch, (int)blocks, scratch + kRedBlocks);
+    k_xsec_final<<<nb, kRedThreads, 0, st>>>(part, (int)blocks, scratch);
     DDA_LAUNCH_CHECK("cross-section final sum");
     return 0;
 }
@@ -412,9 +510,9 @@ int launch_csca(const TargetView& tv, const Geometry& g, double k, const double2
                 const double2* AP, const double2* AhP, double2* scratch, cudaStream_t st) {
     const unsigned blocks =
         (unsigned)std::min<int64_t>(kRedBlocks, std::max<int64_t>(1, (g.nsites + kRedThreads - 1) / kRedThreads));
-    k_csca_partial<<<blocks, kRedThreads, 0, st>>>(tv, g, k * k * k, ainv, P, AP, AhP, scratch);
+    k_csca_partial<<<blocks, kRedThreads, 0, st>>>(tv, g, k * k * k, ainv, P, AP, AhP, scratch + kXsecBatch);
     DDA_LAUNCH_CHECK("C_sca partial sums");
-    k_xsec_final<<<1, kRedThreads, 0, st>>>(scratch, (int)blocks, scratch + kRedBlocks);
+    k_xsec_final<<<1, kRedThreads, 0, st>>>(scratch + kXsecBatch, (int)blocks, scratch);
     DDA_LAUNCH_CHECK("C_sca final sum");
     return 0;
 }

@@ -31,13 +31,16 @@ int launch_site_ranks(const TargetView& tv, int64_t n, uint32_t* out, cudaStream
 int launch_incident(const TargetView& tv, const Geometry& g, double k, const double* khat, const double* e0,
                     double2* E, cudaStream_t st);
 
+// right-hand sides of one launch_cross_sections call (at most)
+constexpr int kXsecBatch = 32;
 size_t xsec_scratch_elems();
-// scratch[xsec_scratch_elems()-1] receives {sum Im(E^* P), sum [-Im ainv - 2/3 k^3] |P|^2}
-int launch_cross_sections(const TargetView& tv, const Geometry& g, double k, const double2* ainv,
+// scratch[b] receives {sum Im(E_b^* P_b), sum [-Im ainv - 2/3 k^3] |P_b|^2} for b < nb <= kXsecBatch
+// (E, P: [nb][3][N_d])
+int launch_cross_sections(const TargetView& tv, const Geometry& g, double k, const double2* ainv, int nb,
                           const double2* E, const double2* P, double2* scratch, cudaStream_t st);
 
 // C_sca by the exact pair sum from P, A P and A^H P; the sum lands in
-// scratch[xsec_scratch_elems()-1].x (without the 4 pi k factor)
+// scratch[0].x (without the 4 pi k factor)
 int launch_csca(const TargetView& tv, const Geometry& g, double k, const double2* ainv, const double2* P,
                 const double2* AP, const double2* AhP, double2* scratch, cudaStream_t st);
 // which: 0 = C_ext, 1 = C_abs

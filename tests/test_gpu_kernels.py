@@ -1,0 +1,62 @@
+"""Kernels at the edges of their ranges (tile remainders, chunk borders, the
+smallest and largest sizes of a dispatch rule) against the FP64 oracle or
+against the general path, through the C ABI."""
+import numpy as np
+import pytest
+
+import synth
+from oracle import dda as odda
+
+from _cases import Case, random_case
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+DEV = "cuda"
+EPS = 2.0 ** -53
+
+
+@pytest.fixture(scope="module")
+def dda():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_0908_0863_gb300 as m
+    return m
+
+
+# ------------------------------------------------ incident field, cross sections
+
+# rows of 1 to 512 sites (the unrolled x loop takes 128 at a time), and
+# 40,000 rows (more than one CTA round of 128 rows x 304 CTAs)
+@pytest.mark.parametrize("shape,fill", [((1, 1, 1), 1.0), ((129, 3, 2), 0.5), ((512, 2, 3), 0.3), ((33, 17, 5), 0.6),
+                                        ((3, 200, 200), 0.4)])
+def test_incident_field_edges(dda, shape, fill):
+    case = random_case(shape, seed=sum(shape), fill=fill, two_materials=False)
+    kh = synth.random_direction(7)[0]
+    e = np.array([0.3 + 0.1j, -0.5j, 0.7])
+    with case.lattice() as lat:
+        E = torch.empty((3, case.nd), dtype=torch.complex128, device=DEV)
+        lat.incident_field(kh, e, E)
+        ref = odda.incident_field(case.coords, case.k, kh, e)
+        # the phase is an FP64 angle of up to k sum(n): its own rounding on
+        # both sides (three products and sums), plus the complex products
+        bound = 8 * EPS * (1.0 + case.k * sum(shape))
+        assert np.abs(E.cpu().numpy() - ref).max() <= bound * np.abs(e).sum()
+
+
+# right-hand sides below, at and above the 32 of one launch
+@pytest.mark.parametrize("two", [False, True])
+@pytest.mark.parametrize("nb", [1, 32, 33, 70])
+def test_cross_sections_batches(dda, nb, two):
+    case = random_case((9, 7, 11), seed=nb, fill=0.7, two_materials=two)
+    E = synth.complex_normal(nb, (nb, 3, case.nd))
+    P = (0.2 - 0.1j) * E + 0.05 * synth.complex_normal(nb + 1, (nb, 3, case.nd))
+    with case.lattice() as lat:
+        got = lat.cross_sections_batch(torch.from_numpy(E).to(DEV), torch.from_numpy(P).to(DEV))
+    for b in range(nb):
+        ext, ab = odda.c_ext(E[b], P[b], case.k), odda.c_abs(case.ainv, P[b], case.k)
+        # sums of 3 N_d terms of either sign: their rounding is below N_d eps times the sum of their sizes
+        f = 4 * np.pi * case.k * EPS * 6 * case.nd
+        w = np.abs(case.ainv.T.imag) + case.k**3
+        assert abs(got[b, 0] - ext) <= f * np.abs(E[b] * P[b]).sum()
+        assert abs(got[b, 1] - ab) <= f * (w * np.abs(P[b]) ** 2).sum()
+        assert got[b, 2] == got[b, 0] - got[b, 1]
