@@ -107,6 +107,7 @@ template <typename T, int N, int LOGW>
 __global__ void __launch_bounds__(kYThreads) k_p1(MatvecView<T> mv, const C<IO<T>>* __restrict__ p) {
     // the three components of a site share its occupancy and rank lookup:
     // each thread gathers all three and transforms them as three lines
+    if (!grid_begin()) return;
     const int j = blockIdx.z;                                  // batch slot
     const int b = mv.b0 + j;
     if (rhs_done(mv, b)) return;
@@ -201,6 +202,7 @@ __global__ void __launch_bounds__(rows_max_threads(N, sizeof(T) == 8)) k_rows(Ma
     const int c = blockIdx.z % 3, j = blockIdx.z / 3;      // component, batch slot
     if (rhs_done(mv, mv.b0 + j)) return;
     extern __shared__ unsigned char smem_raw[];
+    if (!grid_begin()) return;
     using MP = Map<T, N>;
     constexpr int TL = MP::T_, V = MP::V, nv = MP::NV, nh = MP::NH, Wz = 1 << LOGZ;
     constexpr int G = rows_groups(N, Wz, sizeof(T) == 8);
@@ -326,6 +328,7 @@ __global__ void __launch_bounds__(p3_max_threads<T>(N)) k_p3(MatvecView<T> mv) {
     const int j = blockIdx.x;                                   // batch slot
     if (rhs_done(mv, mv.b0 + j)) return;
     extern __shared__ unsigned char smem_raw[];
+    if (!grid_begin()) return;
     C<T>* sm = reinterpret_cast<C<T>*>(smem_raw);
     constexpr int TL = Line<N>::T, nv = Line<N>::NV;
     const Geometry& g = mv.g;
@@ -410,6 +413,7 @@ __global__ void __launch_bounds__(p3_max_threads<T>(N)) __maxnreg__(sizeof(T) ==
     const int j = blockIdx.x;                                   // batch slot
     if (rhs_done(mv, mv.b0 + j)) return;
     extern __shared__ unsigned char smem_raw[];
+    if (!grid_begin()) return;
     C<T>* sm = reinterpret_cast<C<T>*>(smem_raw);
     constexpr int TL = Wide<N>::T, V = Wide<N>::V, nh = V / 2;
     constexpr int KP = 10;                                      // key of the product exchange (no pad)
@@ -488,6 +492,7 @@ __global__ void __launch_bounds__(kYThreads, sizeof(T) == 4 ? 2 : 1) k_p5(Matvec
     const int c = blockIdx.z % 3, j = blockIdx.z / 3;      // component, batch slot
     const int b = mv.b0 + j;
     if (rhs_done(mv, b)) return;
+    if (!grid_begin()) return;
     extern __shared__ unsigned char smem_raw[];
     C<T>* sm = reinterpret_cast<C<T>*>(smem_raw);
     constexpr int TL = Line<N>::T, nv = Line<N>::NV;
@@ -574,7 +579,7 @@ int launch_p1(const MatvecView<T>& mv, const C<IO<T>>* p, cudaStream_t st) {
     static std::atomic<size_t> smem_set{0};
     if (int rc = set_smem((const void*)k_p1<T, N, LOGW>, sm, smem_set)) return rc;
     dim3 grid((g.K + W - 1) / W, g.P, mv.nb);
-    k_p1<T, N, LOGW><<<grid, W * Line<N>::T, sm, st>>>(mv, p);
+    launch_after(k_p1<T, N, LOGW>, grid, W * Line<N>::T, sm, st, mv, p);
     DDA_LAUNCH_CHECK("P1 expand + y-forward");
     return 0;
 }
@@ -594,7 +599,7 @@ int launch_rows_w(const MatvecView<T>& mv, cudaStream_t st) {
         static std::atomic<size_t> smem_set{0};
         if (int rc = set_smem((const void*)k_rows<T, INV, N, LOGZ>, sm, smem_set)) return rc;
         const dim3 grid((unsigned)((g.P + G * Wz - 1) / (G * Wz)), g.Ly, 3 * mv.nb);
-        k_rows<T, INV, N, LOGZ><<<grid, threads, sm, st>>>(mv);
+        launch_after(k_rows<T, INV, N, LOGZ>, grid, threads, sm, st, mv);
         DDA_LAUNCH_CHECK(INV ? "P4 x-inverse" : "P2 x-forward");
         return 0;
     }
@@ -621,10 +626,10 @@ int launch_p3(const MatvecView<T>& mv, cudaStream_t st) {
     const dim3 grid(mv.nb, (g.Lx + R - 1) / R, g.Ly);
     if constexpr (Line<N>::ODD) {   // the wide z pass for 3 * 2^a and 5 * 2^a columns
         if (int rc = set_smem((const void*)k_p3w<T, N>, sm, smem_set)) return rc;
-        k_p3w<T, N><<<grid, R * p3_col_threads(N), sm, st>>>(mv);
+        launch_after(k_p3w<T, N>, grid, R * p3_col_threads(N), sm, st, mv);
     } else {
         if (int rc = set_smem((const void*)k_p3<T, N>, sm, smem_set)) return rc;
-        k_p3<T, N><<<grid, R * p3_col_threads(N), sm, st>>>(mv);
+        launch_after(k_p3<T, N>, grid, R * p3_col_threads(N), sm, st, mv);
     }
     DDA_LAUNCH_CHECK("P3 z-forward, spectrum product, z-inverse");
     return 0;
@@ -638,7 +643,7 @@ int launch_p5(const MatvecView<T>& mv, const C<IO<T>>* p, C<IO<T>>* y, cudaStrea
     static std::atomic<size_t> smem_set{0};
     if (int rc = set_smem((const void*)k_p5<T, N, LOGW>, sm, smem_set)) return rc;
     dim3 grid((g.K + W - 1) / W, g.P, 3 * mv.nb);
-    k_p5<T, N, LOGW><<<grid, W * Line<N>::T, sm, st>>>(mv, p, y);
+    launch_after(k_p5<T, N, LOGW>, grid, W * Line<N>::T, sm, st, mv, p, y);
     DDA_LAUNCH_CHECK("P5 y-inverse + diagonal + compress");
     return 0;
 }

@@ -60,3 +60,37 @@ def test_cross_sections_batches(dda, nb, two):
         assert abs(got[b, 0] - ext) <= f * np.abs(E[b] * P[b]).sum()
         assert abs(got[b, 1] - ab) <= f * (w * np.abs(P[b]) ** 2).sum()
         assert got[b, 2] == got[b, 0] - got[b, 1]
+
+
+# ------------------------------------------------------ dependent launches
+
+# products queued back to back with other work of the same stream between
+# them, on the current stream and on another one: the passes may be scheduled
+# early but must see all earlier writes
+@pytest.mark.parametrize("side", [False, True])
+@pytest.mark.parametrize("shape", [(6, 5, 4), (40, 24, 33)])
+def test_products_in_stream_order(dda, shape, side):
+    case = random_case(shape, seed=3, fill=0.8)
+    with case.lattice() as lat:
+        p0 = torch.from_numpy(synth.complex_normal(5, (3, case.nd), np.complex64)).to(DEV)
+        torch.cuda.synchronize()
+        want, p = [], p0.clone()
+        for _ in range(6):
+            y = torch.empty_like(p)
+            lat.matvec(p, y)
+            torch.cuda.synchronize()
+            want.append(y.clone())
+            p = y * 0.25
+            torch.cuda.synchronize()
+        stream = torch.cuda.Stream() if side else torch.cuda.current_stream()
+        with torch.cuda.stream(stream):
+            got, p = [], p0.clone()
+            for _ in range(6):
+                y = torch.empty_like(p)
+                lat.matvec(p, y)
+                got.append(y.clone())
+                p = y * 0.25
+        stream.synchronize()
+        for a, b in zip(got, want):
+            assert torch.equal(a, b)
+
