@@ -199,10 +199,10 @@ __host__ __device__ constexpr int rows_tile_elems(int N, int Wz, bool c128) {
 
 template <typename T, bool INV, int N, int LOGZ>
 __global__ void __launch_bounds__(rows_max_threads(N, sizeof(T) == 8)) k_rows(MatvecView<T> mv) {
+    if (!grid_begin()) return;
     const int c = blockIdx.z % 3, j = blockIdx.z / 3;      // component, batch slot
     if (rhs_done(mv, mv.b0 + j)) return;
     extern __shared__ unsigned char smem_raw[];
-    if (!grid_begin()) return;
     using MP = Map<T, N>;
     constexpr int TL = MP::T_, V = MP::V, nv = MP::NV, nh = MP::NH, Wz = 1 << LOGZ;
     constexpr int G = rows_groups(N, Wz, sizeof(T) == 8);
@@ -325,10 +325,10 @@ __device__ __forceinline__ void put_line(C<T> (&v)[3][8], int c, const C<T> (&u)
 // DFTs, and the store of k < P.  Grid: (nb, Lx / R, Ly).
 template <typename T, int N>
 __global__ void __launch_bounds__(p3_max_threads<T>(N)) k_p3(MatvecView<T> mv) {
+    if (!grid_begin()) return;
     const int j = blockIdx.x;                                   // batch slot
     if (rhs_done(mv, mv.b0 + j)) return;
     extern __shared__ unsigned char smem_raw[];
-    if (!grid_begin()) return;
     C<T>* sm = reinterpret_cast<C<T>*>(smem_raw);
     constexpr int TL = Line<N>::T, nv = Line<N>::NV;
     const Geometry& g = mv.g;
@@ -410,10 +410,10 @@ __global__ void __launch_bounds__(p3_max_threads<T>(N)) k_p3(MatvecView<T> mv) {
 template <typename T, int N>
 __global__ void __launch_bounds__(p3_max_threads<T>(N)) __maxnreg__(sizeof(T) == 4 ? 128 : 255) k_p3w(MatvecView<T> mv) {
     static_assert(Line<N>::ODD, "k_p3w takes 3 * 2^a and 5 * 2^a columns (their spectrum lines are [6][Hz])");
+    if (!grid_begin()) return;
     const int j = blockIdx.x;                                   // batch slot
     if (rhs_done(mv, mv.b0 + j)) return;
     extern __shared__ unsigned char smem_raw[];
-    if (!grid_begin()) return;
     C<T>* sm = reinterpret_cast<C<T>*>(smem_raw);
     constexpr int TL = Wide<N>::T, V = Wide<N>::V, nh = V / 2;
     constexpr int KP = 10;                                      // key of the product exchange (no pad)
@@ -489,10 +489,10 @@ __global__ void __launch_bounds__(p3_max_threads<T>(N)) __maxnreg__(sizeof(T) ==
 // ---------------------------------------------------------------- P5
 template <typename T, int N, int LOGW>
 __global__ void __launch_bounds__(kYThreads, sizeof(T) == 4 ? 2 : 1) k_p5(MatvecView<T> mv, const C<IO<T>>* __restrict__ p, C<IO<T>>* __restrict__ y) {
+    if (!grid_begin()) return;
     const int c = blockIdx.z % 3, j = blockIdx.z / 3;      // component, batch slot
     const int b = mv.b0 + j;
     if (rhs_done(mv, b)) return;
-    if (!grid_begin()) return;
     extern __shared__ unsigned char smem_raw[];
     C<T>* sm = reinterpret_cast<C<T>*>(smem_raw);
     constexpr int TL = Line<N>::T, nv = Line<N>::NV;
