@@ -588,7 +588,7 @@ int dda_init_lattice(dda_ctx** out, const int32_t shape[3], const uint32_t* occu
         // double-float copies (each double split into a float and the rounded remainder)
         auto split = [](const std::vector<double2>& v) {
             std::vector<cdf> out(v.size());
-            for (size_t i = 0; i < v.size(); ++i) { out[i].x = DF(v[i].x); out[i].y = DF(v[i].y); }
+            for (size_t i = 0; i < v.size(); ++i) out[i] = make_cdf(DF(v[i].x), DF(v[i].y));
             return out;
         };
         const std::vector<cdf> aidf = split(ai), sjdf = split(sj), twdf = split(t64);

@@ -23,42 +23,53 @@ template <typename T> using C = typename cpx<T>::t;
 template <typename T> struct io_of { using t = T; };
 template <> struct io_of<DF> { using t = double; };
 template <typename T> using IO = typename io_of<T>::t;
-template <typename T> __host__ __device__ __forceinline__ C<T> from_io(C<IO<T>> v) { return v; }
-template <> __host__ __device__ __forceinline__ cdf from_io<DF>(double2 v) {
-    cdf z;
-    z.x = DF(v.x);
-    z.y = DF(v.y);
-    return z;
-}
-template <typename T> __host__ __device__ __forceinline__ C<IO<T>> to_io(C<T> v) { return v; }
-template <> __host__ __device__ __forceinline__ double2 to_io<DF>(cdf v) {
-    return make_double2(to_double(v.x), to_double(v.y));
+template <typename T> __device__ __forceinline__ C<T> from_io(C<IO<T>> v) { return v; }
+template <> __device__ __forceinline__ cdf from_io<DF>(double2 v) { return make_cdf(df_split(v.x), df_split(v.y)); }
+template <typename T> __device__ __forceinline__ C<IO<T>> to_io(C<T> v) { return v; }
+template <> __device__ __forceinline__ double2 to_io<DF>(cdf v) {
+    return make_double2(df_widen(v.h.x) + df_widen(v.l.x), df_widen(v.h.y) + df_widen(v.l.y));
 }
 // read-only cached load of one complex value
 template <typename T> __device__ __forceinline__ C<T> ldg_c(const C<T>* p) { return __ldg(p); }
 template <> __device__ __forceinline__ cdf ldg_c<DF>(const cdf* p) {
     const float4 f = __ldg(reinterpret_cast<const float4*>(p));
-    cdf z;
-    z.x = DF(f.x, f.y);
-    z.y = DF(f.z, f.w);
-    return z;
+    return cdf{make_float2(f.x, f.y), make_float2(f.z, f.w)};
 }
 
 template <typename T> __host__ __device__ __forceinline__ C<T> mk(T re, T im) { C<T> z; z.x = re; z.y = im; return z; }
-template <typename T> __host__ __device__ __forceinline__ C<T> cadd(C<T> a, C<T> b) { return mk<T>(a.x + b.x, a.y + b.y); }
-template <typename T> __host__ __device__ __forceinline__ C<T> csub(C<T> a, C<T> b) { return mk<T>(a.x - b.x, a.y - b.y); }
-template <typename T> __host__ __device__ __forceinline__ C<T> cmul(C<T> a, C<T> b) {
+template <typename T> __device__ __forceinline__ C<T> cadd(C<T> a, C<T> b) { return mk<T>(a.x + b.x, a.y + b.y); }
+template <typename T> __device__ __forceinline__ C<T> csub(C<T> a, C<T> b) { return mk<T>(a.x - b.x, a.y - b.y); }
+template <typename T> __device__ __forceinline__ C<T> cmul(C<T> a, C<T> b) {
     return mk<T>(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }
 // a * conj(b)
-template <typename T> __host__ __device__ __forceinline__ C<T> cmulc(C<T> a, C<T> b) {
+template <typename T> __device__ __forceinline__ C<T> cmulc(C<T> a, C<T> b) {
     return mk<T>(a.x * b.x + a.y * b.y, a.y * b.x - a.x * b.y);
 }
-template <typename T> __host__ __device__ __forceinline__ C<T> cscale(C<T> a, T s) { return mk<T>(a.x * s, a.y * s); }
+template <typename T> __device__ __forceinline__ C<T> cscale(C<T> a, T s) { return mk<T>(a.x * s, a.y * s); }
+template <typename T> __device__ __forceinline__ C<T> cneg(C<T> a) { return mk<T>(-a.x, -a.y); }
+template <typename T> __device__ __forceinline__ C<T> cconj(C<T> a) { return mk<T>(a.x, -a.y); }
 // acc += a * b
-template <typename T> __host__ __device__ __forceinline__ C<T> cfma(C<T> a, C<T> b, C<T> acc) {
+template <typename T> __device__ __forceinline__ C<T> cfma(C<T> a, C<T> b, C<T> acc) {
     return mk<T>(fma(a.x, b.x, fma(-a.y, b.y, acc.x)), fma(a.x, b.y, fma(a.y, b.x, acc.y)));
 }
+// a x + b y + c z
+template <typename T> __device__ __forceinline__ C<T> cdot3(C<T> a, C<T> x, C<T> b, C<T> y, C<T> c, C<T> z) {
+    return cfma<T>(c, z, cfma<T>(b, y, cmul<T>(a, x)));
+}
+// the double-float forms (pairs of high and low parts, df.cuh)
+template <> __host__ __device__ __forceinline__ cdf mk<DF>(DF re, DF im) { return make_cdf(re, im); }
+template <> __device__ __forceinline__ cdf cadd<DF>(cdf a, cdf b) { return df_add(a, b); }
+template <> __device__ __forceinline__ cdf csub<DF>(cdf a, cdf b) { return df_sub(a, b); }
+template <> __device__ __forceinline__ cdf cmul<DF>(cdf a, cdf b) { return df_cmul(a, b); }
+template <> __device__ __forceinline__ cdf cscale<DF>(cdf a, DF s) { return df_cscale(a, s); }
+template <> __device__ __forceinline__ cdf cneg<DF>(cdf a) {
+    return cdf{make_float2(-a.h.x, -a.h.y), make_float2(-a.l.x, -a.l.y)};
+}
+template <> __device__ __forceinline__ cdf cconj<DF>(cdf a) {
+    return cdf{make_float2(a.h.x, -a.h.y), make_float2(a.l.x, -a.l.y)};
+}
+template <> __device__ __forceinline__ cdf cfma<DF>(cdf a, cdf b, cdf acc) { return df_cfma(a, b, acc); }
 
 // --------------------------------------------------------------- limits
 constexpr int kTwEntries = 3072 + 5120;   // twiddle tables exp(-2 pi i m / 3072) and exp(-2 pi i m / 5120)

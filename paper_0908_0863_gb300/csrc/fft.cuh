@@ -29,6 +29,26 @@ template <typename T, bool INV>
 __device__ __forceinline__ C<T> rot90(C<T> a) {  // times -i (forward) or +i (inverse)
     return INV ? mk<T>(-a.y, a.x) : mk<T>(a.y, -a.x);
 }
+template <> __device__ __forceinline__ cdf rot90<DF, true>(cdf a) { return cdf{turned(a.h), turned(a.l)}; }
+template <> __device__ __forceinline__ cdf rot90<DF, false>(cdf a) {
+    return cdf{make_float2(a.h.y, -a.h.x), make_float2(a.l.y, -a.l.x)};
+}
+
+// times exp(-+ 2 pi i / 8) and exp(-+ 2 pi i 3 / 8) (forward -, inverse +)
+template <typename T, bool INV>
+__device__ __forceinline__ C<T> turn8(C<T> b) {
+    const T h = (T)0.70710678118654752440;  // 1/sqrt(2)
+    return INV ? mk<T>((b.x - b.y) * h, (b.x + b.y) * h) : mk<T>((b.x + b.y) * h, (b.y - b.x) * h);
+}
+template <typename T, bool INV>
+__device__ __forceinline__ C<T> turn83(C<T> b) {
+    const T h = (T)0.70710678118654752440;
+    return INV ? mk<T>((-b.x - b.y) * h, (b.x - b.y) * h) : mk<T>((b.y - b.x) * h, (-b.x - b.y) * h);
+}
+template <> __device__ __forceinline__ cdf turn8<DF, false>(cdf b) { return df_cscale(df_add(b, rot90<DF, false>(b)), DF(0.70710678118654752440)); }
+template <> __device__ __forceinline__ cdf turn8<DF, true>(cdf b) { return df_cscale(df_add(b, rot90<DF, true>(b)), DF(0.70710678118654752440)); }
+template <> __device__ __forceinline__ cdf turn83<DF, false>(cdf b) { return df_cscale(df_sub(rot90<DF, false>(b), b), DF(0.70710678118654752440)); }
+template <> __device__ __forceinline__ cdf turn83<DF, true>(cdf b) { return df_cscale(df_sub(rot90<DF, true>(b), b), DF(0.70710678118654752440)); }
 
 template <typename T, bool INV>
 __device__ __forceinline__ void dft2(C<T>* v) {
@@ -52,7 +72,6 @@ __device__ __forceinline__ void dft4(C<T>* v) {
 // twiddles W8^r, then two radix-4 DFTs on the even and odd outputs
 template <typename T, bool INV>
 __device__ __forceinline__ void dft8(C<T>* v) {
-    const T h = (T)0.70710678118654752440;  // 1/sqrt(2)
     C<T> a[4], b[4];
 #pragma unroll
     for (int r = 0; r < 4; ++r) {
@@ -60,13 +79,8 @@ __device__ __forceinline__ void dft8(C<T>* v) {
         b[r] = csub<T>(v[r], v[r + 4]);
     }
     // b1 *= W8^1, b2 *= W8^2, b3 *= W8^3 (conjugated for the inverse)
-    if (INV) {
-        b[1] = mk<T>((b[1].x - b[1].y) * h, (b[1].x + b[1].y) * h);
-        b[3] = mk<T>((-b[3].x - b[3].y) * h, (b[3].x - b[3].y) * h);
-    } else {
-        b[1] = mk<T>((b[1].x + b[1].y) * h, (b[1].y - b[1].x) * h);
-        b[3] = mk<T>((b[3].y - b[3].x) * h, (-b[3].x - b[3].y) * h);
-    }
+    b[1] = turn8<T, INV>(b[1]);
+    b[3] = turn83<T, INV>(b[3]);
     b[2] = rot90<T, INV>(b[2]);
     dft4<T, INV>(a);
     dft4<T, INV>(b);

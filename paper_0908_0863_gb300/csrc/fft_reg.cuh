@@ -51,6 +51,8 @@
 // and form the others as its powers.  Transforms are unnormalised.
 #pragma once
 
+#include <type_traits>
+
 #include "fft.cuh"
 
 namespace dda {
@@ -210,25 +212,18 @@ __host__ __device__ constexpr int col_elems(int N, int W) { return col_elems_sh(
 
 template <typename T, bool INV>
 __device__ __forceinline__ C<T> twiddle(const C<T>* __restrict__ tw, int idx) {
-    C<T> t = ldg_c<T>(tw + idx);
-    if (INV) t.y = -t.y;
-    return t;
+    const C<T> t = ldg_c<T>(tw + idx);
+    return INV ? cconj<T>(t) : t;
 }
 
 // radix-8 DFT with inputs 4..7 known to be zero: the first layer of dft8
 // degenerates to copies
 template <typename T, bool INV>
 __device__ __forceinline__ void dft8_half_in(C<T>* v) {
-    const T h = (T)0.70710678118654752440;
     C<T> a[4] = {v[0], v[1], v[2], v[3]};
     C<T> b[4] = {v[0], v[1], v[2], v[3]};
-    if (INV) {
-        b[1] = mk<T>((b[1].x - b[1].y) * h, (b[1].x + b[1].y) * h);
-        b[3] = mk<T>((-b[3].x - b[3].y) * h, (b[3].x - b[3].y) * h);
-    } else {
-        b[1] = mk<T>((b[1].x + b[1].y) * h, (b[1].y - b[1].x) * h);
-        b[3] = mk<T>((b[3].y - b[3].x) * h, (-b[3].x - b[3].y) * h);
-    }
+    b[1] = turn8<T, INV>(b[1]);
+    b[3] = turn83<T, INV>(b[3]);
     b[2] = rot90<T, INV>(b[2]);
     dft4<T, INV>(a);
     dft4<T, INV>(b);
@@ -242,20 +237,14 @@ __device__ __forceinline__ void dft8_half_in(C<T>* v) {
 // radix-8 DFT computing only outputs 0..3 (outputs 4..7 left unspecified)
 template <typename T, bool INV>
 __device__ __forceinline__ void dft8_half_out(C<T>* v) {
-    const T h = (T)0.70710678118654752440;
     C<T> a[4], b[4];
 #pragma unroll
     for (int r = 0; r < 4; ++r) {
         a[r] = cadd<T>(v[r], v[r + 4]);
         b[r] = csub<T>(v[r], v[r + 4]);
     }
-    if (INV) {
-        b[1] = mk<T>((b[1].x - b[1].y) * h, (b[1].x + b[1].y) * h);
-        b[3] = mk<T>((-b[3].x - b[3].y) * h, (b[3].x - b[3].y) * h);
-    } else {
-        b[1] = mk<T>((b[1].x + b[1].y) * h, (b[1].y - b[1].x) * h);
-        b[3] = mk<T>((b[3].y - b[3].x) * h, (-b[3].x - b[3].y) * h);
-    }
+    b[1] = turn8<T, INV>(b[1]);
+    b[3] = turn83<T, INV>(b[3]);
     b[2] = rot90<T, INV>(b[2]);
     // outputs 0, 2 from the even radix-4 (its outputs 0, 1), 1, 3 from the odd
     const C<T> ca0 = cadd<T>(a[0], a[2]), ca2 = csub<T>(a[0], a[2]);
@@ -309,7 +298,9 @@ template <typename T, bool INV>
 __device__ __forceinline__ void dft3(C<T>& a, C<T>& b, C<T>& c) {
     const T h = (T)0.86602540378443864676;   // sqrt(3) / 2
     const C<T> s = cadd<T>(b, c), d = csub<T>(b, c);
-    const C<T> m = mk<T>(a.x - (T)0.5 * s.x, a.y - (T)0.5 * s.y);
+    C<T> m;
+    if constexpr (std::is_same<T, DF>::value) m = csub<DF>(a, cdf{__fmul2_rn(s.h, both(0.5f)), __fmul2_rn(s.l, both(0.5f))});
+    else m = mk<T>(a.x - (T)0.5 * s.x, a.y - (T)0.5 * s.y);
     const C<T> r = cscale<T>(rot90<T, INV>(d), h);
     a = cadd<T>(a, s);
     b = cadd<T>(m, r);
@@ -323,10 +314,18 @@ __device__ __forceinline__ void dft5(C<T> (&x)[5]) {
     const T s1 = (T)0.95105651629515357212, s2 = (T)0.58778525229247312917;    // sin(2 pi/5), sin(4 pi/5)
     const C<T> a1 = cadd<T>(x[1], x[4]), b1 = csub<T>(x[1], x[4]);
     const C<T> a2 = cadd<T>(x[2], x[3]), b2 = csub<T>(x[2], x[3]);
-    const C<T> t1 = mk<T>(x[0].x + c1 * a1.x + c2 * a2.x, x[0].y + c1 * a1.y + c2 * a2.y);
-    const C<T> t2 = mk<T>(x[0].x + c2 * a1.x + c1 * a2.x, x[0].y + c2 * a1.y + c1 * a2.y);
-    const C<T> u1 = rot90<T, INV>(mk<T>(s1 * b1.x + s2 * b2.x, s1 * b1.y + s2 * b2.y));
-    const C<T> u2 = rot90<T, INV>(mk<T>(s2 * b1.x - s1 * b2.x, s2 * b1.y - s1 * b2.y));
+    C<T> t1, t2, u1, u2;
+    if constexpr (std::is_same<T, DF>::value) {
+        t1 = cadd<DF>(cadd<DF>(x[0], cscale<DF>(a1, c1)), cscale<DF>(a2, c2));
+        t2 = cadd<DF>(cadd<DF>(x[0], cscale<DF>(a1, c2)), cscale<DF>(a2, c1));
+        u1 = rot90<DF, INV>(cadd<DF>(cscale<DF>(b1, s1), cscale<DF>(b2, s2)));
+        u2 = rot90<DF, INV>(csub<DF>(cscale<DF>(b1, s2), cscale<DF>(b2, s1)));
+    } else {
+        t1 = mk<T>(x[0].x + c1 * a1.x + c2 * a2.x, x[0].y + c1 * a1.y + c2 * a2.y);
+        t2 = mk<T>(x[0].x + c2 * a1.x + c1 * a2.x, x[0].y + c2 * a1.y + c1 * a2.y);
+        u1 = rot90<T, INV>(mk<T>(s1 * b1.x + s2 * b2.x, s1 * b1.y + s2 * b2.y));
+        u2 = rot90<T, INV>(mk<T>(s2 * b1.x - s1 * b2.x, s2 * b1.y - s1 * b2.y));
+    }
     x[0] = cadd<T>(x[0], cadd<T>(a1, a2));
     x[1] = cadd<T>(t1, u1);
     x[4] = csub<T>(t1, u1);
@@ -580,13 +579,18 @@ __device__ __forceinline__ C<T> cmul_root(C<T> x, int e) {
     if (e < 0) e += V;
     if (e == 0) return x;
     if (4 * e == V) return rot90<T, INV>(x);
-    if (2 * e == V) return mk<T>(-x.x, -x.y);
+    if (2 * e == V) return cneg<T>(x);
     if (4 * e == 3 * V) return rot90<T, !INV>(x);
     if ((8 * e) % V == 0) {   // (+-1 +- i) / sqrt(2)
         const T h = (T)0.70710678118654752440;
         const double cr = cos_v<V>(e), sr = INV ? cos_v<V>(e - V / 4) : -cos_v<V>(e - V / 4);
+        if constexpr (std::is_same<T, DF>::value) {
+            const cdf p = cr > 0 ? x : cneg<DF>(x), q = sr > 0 ? rot90<DF, true>(x) : rot90<DF, false>(x);
+            return cscale<DF>(cadd<DF>(p, q), h);
+        } else {
         const T c = (T)(cr > 0 ? 1.0 : -1.0), s = (T)(sr > 0 ? 1.0 : -1.0);
         return mk<T>((c * x.x - s * x.y) * h, (c * x.y + s * x.x) * h);
+        }
     }
     return cmul<T>(x, root_v<T, INV, V>(e));
 }

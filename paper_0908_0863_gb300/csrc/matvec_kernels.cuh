@@ -149,7 +149,7 @@ __global__ void __launch_bounds__(kYThreads) k_p1(MatvecView<T> mv, const C<IO<T
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
                 v[c][m] = from_io<T>(pb[c * g.nd + r]);
-                if (mv.conj) v[c][m].y = -v[c][m].y;
+                if (mv.conj) v[c][m] = cconj<T>(v[c][m]);
             }
         }
     }
@@ -293,11 +293,11 @@ __device__ __forceinline__ void p3_product(const C<T>* __restrict__ line, bool o
     }
 #pragma unroll
     for (int q = 0; q < 6; ++q)
-        if (mirror_flip(q, fx, fy, fz)) { Y[q].x = -Y[q].x; Y[q].y = -Y[q].y; }
+        if (mirror_flip(q, fx, fy, fz)) Y[q] = cneg<T>(Y[q]);
     const C<T> a = X0, b = X1, c = X2;
-    X0 = cfma<T>(Y[2], c, cfma<T>(Y[1], b, cmul<T>(Y[0], a)));
-    X1 = cfma<T>(Y[4], c, cfma<T>(Y[3], b, cmul<T>(Y[1], a)));
-    X2 = cfma<T>(Y[5], c, cfma<T>(Y[4], b, cmul<T>(Y[2], a)));
+    X0 = cdot3<T>(Y[0], a, Y[1], b, Y[2], c);
+    X1 = cdot3<T>(Y[1], a, Y[3], b, Y[4], c);
+    X2 = cdot3<T>(Y[2], a, Y[4], b, Y[5], c);
 }
 
 // Line c of three held in registers, copied out and back with selects on the
@@ -346,7 +346,7 @@ __global__ void __launch_bounds__(p3_max_threads<T>(N)) k_p3(MatvecView<T> mv) {
             v[c][m] = (ok && m < Line<N>::NH && n < g.P) ? col[c * comp + n] : mk<T>(0, 0);
         }
     const int region = row_ld(N, TL) << mv.logW_z;
-    if constexpr (sizeof(T) == 8 && !std::is_same<T, double>::value) {
+    if constexpr (std::is_same<T, DF>::value) {
         // double-float: one component at a time, in a loop that is not
         // unrolled, so that the kernel holds one line's transform instead of
         // three (unrolled, its instruction fetch limited it, not arithmetic)
@@ -368,7 +368,7 @@ __global__ void __launch_bounds__(p3_max_threads<T>(N)) k_p3(MatvecView<T> mv) {
         for (int m = 0; m < nv; ++m)
             p3_product<T, N>(line, ok, fx, fy, t + m * TL, v[0][m], v[1][m], v[2][m]);
     }
-    if constexpr (sizeof(T) == 8 && !std::is_same<T, double>::value) {
+    if constexpr (std::is_same<T, DF>::value) {
         // each transform but the last ends with a barrier after its last
         // shared-memory read, before the next one writes the buffer
 #pragma unroll 1
@@ -456,15 +456,15 @@ __global__ void __launch_bounds__(p3_max_threads<T>(N)) __maxnreg__(sizeof(T) ==
                 const int o0 = L.template at<KP>(3 * w, n), o1 = L.template at<KP>(3 * w + 1, n),
                           o2 = L.template at<KP>(3 * w + 2, n);
                 C<T> a = sm[o0], b = sm[o1], d = sm[o2];
-                if (fx) a = mk<T>(-a.x, -a.y);
-                if (fy) b = mk<T>(-b.x, -b.y);
-                if (fz) d = mk<T>(-d.x, -d.y);
-                C<T> y0 = cfma<T>(G[2], d, cfma<T>(G[1], b, cmul<T>(G[0], a)));
-                C<T> y1 = cfma<T>(G[4], d, cfma<T>(G[3], b, cmul<T>(G[1], a)));
-                C<T> y2 = cfma<T>(G[5], d, cfma<T>(G[4], b, cmul<T>(G[2], a)));
-                if (fx) y0 = mk<T>(-y0.x, -y0.y);
-                if (fy) y1 = mk<T>(-y1.x, -y1.y);
-                if (fz) y2 = mk<T>(-y2.x, -y2.y);
+                if (fx) a = cneg<T>(a);
+                if (fy) b = cneg<T>(b);
+                if (fz) d = cneg<T>(d);
+                C<T> y0 = cdot3<T>(G[0], a, G[1], b, G[2], d);
+                C<T> y1 = cdot3<T>(G[1], a, G[3], b, G[4], d);
+                C<T> y2 = cdot3<T>(G[2], a, G[4], b, G[5], d);
+                if (fx) y0 = cneg<T>(y0);
+                if (fy) y1 = cneg<T>(y1);
+                if (fz) y2 = cneg<T>(y2);
                 sm[o0] = y0;
                 sm[o1] = y1;
                 sm[o2] = y2;
@@ -542,7 +542,7 @@ __global__ void __launch_bounds__(kYThreads, sizeof(T) == 4 ? 2 : 1) k_p5(Matvec
         const int mat = material(mv.tv, s, c);
         const C<T> a = mv.ainv[mat * 3 + c];
         C<T> q = from_io<T>(pv[m]);
-        if (mv.conj) q.y = -q.y;
+        if (mv.conj) q = cconj<T>(q);
         C<T> out;
         if (mv.jac) {   // point-Jacobi: S (alpha^-1 S p + conv)
             const C<T> f = mv.jac[mat * 3 + c];
@@ -550,7 +550,7 @@ __global__ void __launch_bounds__(kYThreads, sizeof(T) == 4 ? 2 : 1) k_p5(Matvec
         } else {
             out = cfma<T>(a, q, v[m]);
         }
-        if (mv.conj) out.y = -out.y;
+        if (mv.conj) out = cconj<T>(out);
         yc[rbase[m]] = to_io<T>(out);
     }
 }

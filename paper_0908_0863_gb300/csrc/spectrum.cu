@@ -248,10 +248,7 @@ __global__ void __launch_bounds__(256) k_spec_export(Geometry g, const C<T>* __r
 __global__ void __launch_bounds__(256) k_spec_to_df(const double2* __restrict__ in, cdf* __restrict__ out, int64_t n) {
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
         const double2 v = in[e];
-        cdf z;
-        z.x = DF(v.x);
-        z.y = DF(v.y);
-        out[e] = z;
+        out[e] = from_io<DF>(v);
     }
 }
 

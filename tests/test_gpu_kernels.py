@@ -94,3 +94,23 @@ def test_products_in_stream_order(dda, shape, side):
         for a, b in zip(got, want):
             assert torch.equal(a, b)
 
+
+# ------------------------------------------------------------ double-float
+
+# vectors around the ends of the range that is split and widened on the
+# integer units (2^-70 .. 2^126), and of both signs with exact zeros
+@pytest.mark.parametrize("exponent", [-90, -71, -70, -66, 0, 60, 100])
+def test_double_float_product_scales(dda, exponent):
+    case = random_case((6, 5, 7), seed=11, fill=0.7)
+    p = synth.complex_normal(12, (3, case.nd))
+    p[:, ::3] = 0.0
+    p[:, 1::3] *= 2.0 ** -20   # entries of two sizes
+    p *= 2.0 ** exponent
+    with case.lattice() as lat:
+        x = torch.from_numpy(p).to(DEV)
+        y, z = torch.empty_like(x), torch.empty_like(x)
+        lat.matvec(x, y)
+        dda.dda_matvec(lat.ctx, x, z, dtype="c128df")
+    # 2^-48 per operation along some 30 operations, on the norm
+    assert float((z - y).norm() / y.norm()) <= 30 * 2.0 ** -48
+
