@@ -62,29 +62,40 @@ struct DotAcc {
     }
 };
 
+// Block sums of NR values per thread.  FP64 additions cost 16 cycles of an
+// SM per warp here, and a shuffle tree in every warp spends most of its lanes
+// on sums nobody reads: the values go through shared memory instead, and warp
+// r adds value r (eight per lane, then one shuffle tree): 24 NR warp-wide
+// additions per block where eight trees take 96 NR.  out(r, sum) runs in one
+// lane per value.
+template <int NR, typename Out>
+__device__ __forceinline__ void block_sums(double2 (&a)[NR], double2 (&sm)[NR][kVecThreads], Out out) {
+#pragma unroll
+    for (int r = 0; r < NR; ++r) sm[r][threadIdx.x] = a[r];
+    __syncthreads();
+    const int lane = threadIdx.x & 31;
+    for (int r = threadIdx.x >> 5; r < NR; r += kVecThreads / 32) {
+        double2 t = sm[r][lane];
+#pragma unroll
+        for (int w = 1; w < kVecThreads / 32; ++w) {
+            const double2 v = sm[r][lane + 32 * w];
+            t.x += v.x;
+            t.y += v.y;
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            t.x += __shfl_down_sync(0xffffffffu, t.x, o);
+            t.y += __shfl_down_sync(0xffffffffu, t.y, o);
+        }
+        if (lane == 0) out(r, t);
+    }
+}
+
 // partial sums of this block into part (already offset to its right-hand side)
 template <int NR>
 __device__ __forceinline__ void block_partials(double2 (&a)[NR], double2* __restrict__ part) {
-    __shared__ double2 sm[NR][kVecThreads / 32];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-    for (int r = 0; r < NR; ++r) {
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            a[r].x += __shfl_down_sync(0xffffffffu, a[r].x, o);
-            a[r].y += __shfl_down_sync(0xffffffffu, a[r].y, o);
-        }
-        if (lane == 0) sm[r][wid] = a[r];
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-#pragma unroll
-        for (int r = 0; r < NR; ++r) {
-            double2 t = make_double2(0.0, 0.0);
-            for (int w = 0; w < kVecThreads / 32; ++w) { t.x += sm[r][w].x; t.y += sm[r][w].y; }
-            part[blockIdx.x * kMaxRed + r] = t;
-        }
-    }
+    __shared__ double2 sm[NR][kVecThreads];
+    block_sums<NR>(a, sm, [&](int r, double2 t) { part[blockIdx.x * kMaxRed + r] = t; });
 }
 
 // all threads of a scalar block call this; every thread gets the sums of
@@ -92,28 +103,21 @@ __device__ __forceinline__ void block_partials(double2 (&a)[NR], double2* __rest
 template <int NR>
 __device__ __forceinline__ void final_sums(const double2* __restrict__ part, int nparts, double2 (&out)[NR]) {
     __shared__ double2 sm[NR][kVecThreads];
+    __shared__ double2 total[NR];
+    double2 a[NR];
 #pragma unroll
-    for (int r = 0; r < NR; ++r) {
-        double2 a = make_double2(0.0, 0.0);
-        for (int i = threadIdx.x; i < nparts; i += blockDim.x) {
-            a.x += part[i * kMaxRed + r].x;
-            a.y += part[i * kMaxRed + r].y;
+    for (int r = 0; r < NR; ++r) a[r] = make_double2(0.0, 0.0);
+    for (int i = threadIdx.x; i < nparts; i += kVecThreads)
+#pragma unroll
+        for (int r = 0; r < NR; ++r) {
+            const double2 v = part[i * kMaxRed + r];
+            a[r].x += v.x;
+            a[r].y += v.y;
         }
-        sm[r][threadIdx.x] = a;
-    }
+    block_sums<NR>(a, sm, [&](int r, double2 t) { total[r] = t; });
     __syncthreads();
-    for (int o = kVecThreads / 2; o > 0; o >>= 1) {
-        if (threadIdx.x < o) {
 #pragma unroll
-            for (int r = 0; r < NR; ++r) {
-                sm[r][threadIdx.x].x += sm[r][threadIdx.x + o].x;
-                sm[r][threadIdx.x].y += sm[r][threadIdx.x + o].y;
-            }
-        }
-        __syncthreads();
-    }
-#pragma unroll
-    for (int r = 0; r < NR; ++r) out[r] = sm[r][0];
+    for (int r = 0; r < NR; ++r) out[r] = total[r];
 }
 
 __device__ __forceinline__ double2 dmul(double2 a, double2 b) { return cmul<double>(a, b); }
