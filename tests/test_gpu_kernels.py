@@ -114,3 +114,18 @@ def test_double_float_product_scales(dda, exponent):
     # 2^-48 per operation along some 30 operations, on the norm
     assert float((z - y).norm() / y.norm()) <= 30 * 2.0 ** -48
 
+
+# short x rows share a CTA for 8-byte reals; z counts that do not fill it
+@pytest.mark.parametrize("K", [1, 2, 4, 7, 16, 32])
+@pytest.mark.parametrize("P", [1, 3, 17])
+def test_short_rows(dda, K, P):
+    case = random_case((K, 3, P), seed=K + P, fill=0.9)
+    p = synth.complex_normal(K * P, (3, case.nd))
+    ref = odda.direct_matvec(case.coords, case.ainv, case.k, p)
+    with case.lattice() as lat:
+        x = torch.from_numpy(p).to(DEV)
+        for dtype, tol in ((None, 1e-13), ("c128df", 1e-12)):
+            y = torch.empty_like(x)
+            dda.dda_matvec(lat.ctx, x, y, dtype=dtype)
+            assert np.abs(y.cpu().numpy() - ref).max() <= tol * np.abs(ref).max()
+
