@@ -612,8 +612,7 @@ int dda_init_lattice(dda_ctx** out, const int32_t shape[3], const uint32_t* occu
         e = cudaMalloc(&tmp, 2 * ns * sizeof(double2));
         if (e != cudaSuccess) return bail(cuda_fail(e, "dda_init_lattice: spectrum scratch"));
         double2* s0 = static_cast<double2*>(tmp);
-        rc = build_spectrum(g, k, c->tw64, s0, s0 + ns, c->spec64, c->spec32, st);
-        if (!rc) rc = spectrum_to_df(c->spec64, c->spec_df, nspec, st);
+        rc = build_spectrum(g, k, c->tw64, s0, s0 + ns, c->spec64, c->spec32, c->spec_df, st);
         cudaError_t e2 = cudaStreamSynchronize(st);
         cudaFree(tmp);
         if (rc) return bail(rc);

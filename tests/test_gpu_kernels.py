@@ -129,3 +129,24 @@ def test_short_rows(dda, K, P):
             dda.dda_matvec(lat.ctx, x, y, dtype=dtype)
             assert np.abs(y.cpu().numpy() - ref).max() <= tol * np.abs(ref).max()
 
+
+# --------------------------------------------------------- tensor spectrum
+
+# paired even and odd lines on every axis, lines of one site among them
+@pytest.mark.parametrize("shape", [(1, 7, 3), (13, 1, 5), (2, 2, 1), (40, 24, 9), (9, 33, 65)])
+def test_tensor_spectrum_pairs(dda, shape):
+    from oracle import circulant
+    K, J, P = shape
+    k = 0.7
+    case = Case(np.ones((P, J, K), dtype=np.uint8), [1.5 + 0.1j], k)
+    L = tuple(circulant.padded_length(v) for v in shape)
+    half = circulant.half_spectrum(circulant.tensor_section1(k, K, J, P), L) / (L[0] * L[1] * L[2])
+    half = np.ascontiguousarray(half.transpose(2, 3, 1, 0))
+    with case.lattice() as lat:
+        out = torch.empty(half.shape, dtype=torch.complex128, device=DEV)
+        lat.tensor_spectrum(out)
+        err = np.abs(out.cpu().numpy() - half)
+    # each component against its own size: a pair shares its rounding, and the
+    # components of a pair are of one size up to the lattice's aspect
+    for q in range(6):
+        assert err[..., q].max() <= 1e-13 * max(np.abs(half[..., q]).max(), 1e-2 * np.abs(half).max())
