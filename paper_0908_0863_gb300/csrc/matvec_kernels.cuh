@@ -489,6 +489,172 @@ __global__ void __launch_bounds__(p3_max_threads<T>(N)) __maxnreg__(sizeof(T) ==
     }
 }
 
+// ------------------------------------------------- P3, split-line mapping
+// The z pass of complex64 columns of 128 points.  Half of each input line is
+// zero and half of each output line is dropped, so the N-point transforms are
+// pairs of N/2 = 64 point ones: the even and the odd frequencies of the
+// forward are the DFTs of x[n] and of x[n] W_N^n, and the kept outputs are the
+// sum of the two inverse DFTs, the odd one times W_N^-n.  A column belongs to
+// 16 lanes of one warp, eight per parity; a lane holds the eight points
+// t + 8 m of all three components, so the spectrum product stays in
+// registers.  A 64-point DFT is a radix-8 stage on the lane's own points, one
+// exchange inside the eight lanes and another radix-8 stage: no barrier of
+// the CTA, and four shared-memory accesses per point where k_p3, which the
+// L1 data pipe bounds, makes eight; one shuffle per kept output joins the
+// parities.  The column's spectrum records come to shared memory
+// asynchronously during the forward transforms.
+// P3 of the 100 x 100 x 60 lattice 92 -> 80 us, of 64^3 26.6 -> 24.8, of a
+// batch of sixteen 64^3 326 -> 283 (unstaged records 314).  Other lengths
+// keep k_p3: 64 points measured 9.3 against 8.1 us; 256 points, as four
+// residues of 64, 180 against 160; 512 points with 16 points per lane, whose
+// 168 registers leave 12 warps on an SM, 1600 against 1310.
+constexpr int kSplitN = 128, kSplitLanes = 16;                  // points and lanes of a column
+// exchange buffers: rows k1 of eight points at pitch 10; the parities' buffers
+// lie 8 elements (mod 16) apart, so that the 8-byte row writes of a half-warp
+// and the 16-byte reads along rows of a quarter meet different banks
+constexpr int kSplitPitch = 10, kSplitBuf = 8 * kSplitPitch + 8;
+constexpr int kSplitSpec = 6 * (kSplitN / 2 + 1);               // spectrum records of a column
+constexpr int kSplitElems = 2 * kSplitBuf + kSplitSpec;         // shared memory of a column
+template <typename T, int N> constexpr bool split_z = std::is_same<T, float>::value && N == kSplitN;
+// columns of a CTA: whole warps
+__host__ __device__ constexpr int split_cols(int R) { return R * kSplitLanes < 32 ? 32 / kSplitLanes : R; }
+
+// forward of one line: v[m] = x[t + 8 m] (times W_N^(8 m) at odd parity) on
+// entry, X[2 (t + 8 k) + h] at v[k] on return; w[i] = W_N^((2 t + h) i)
+__device__ __forceinline__ void split_forward(float2 (&v)[8], float2* __restrict__ sm, int t, const float2 (&w)[8]) {
+    dft8<float, false>(v);
+#pragma unroll
+    for (int k = 0; k < 8; ++k) sm[k * kSplitPitch + t] = v[k];
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < 8; i += 2) {
+        const float4 f = *reinterpret_cast<const float4*>(sm + t * kSplitPitch + i);
+        v[i] = make_float2(f.x, f.y);
+        v[i + 1] = make_float2(f.z, f.w);
+    }
+    __syncwarp();
+#pragma unroll
+    for (int i = 1; i < 8; ++i) v[i] = cmul<float>(v[i], w[i]);
+    dft8<float, false>(v);
+}
+// the inverse: output t + 8 k of the parity's transform at v[k], at odd
+// parity short of the factor W_N^(-8 k)
+__device__ __forceinline__ void split_inverse(float2 (&v)[8], float2* __restrict__ sm, int t, const float2 (&w)[8]) {
+    dft8<float, true>(v);
+#pragma unroll
+    for (int i = 1; i < 8; ++i) v[i] = cmulc<float>(v[i], w[i]);
+#pragma unroll
+    for (int i = 0; i < 8; i += 2)
+        *reinterpret_cast<float4*>(sm + t * kSplitPitch + i) = make_float4(v[i].x, v[i].y, v[i + 1].x, v[i + 1].y);
+    __syncwarp();
+#pragma unroll
+    for (int k = 0; k < 8; ++k) v[k] = sm[k * kSplitPitch + t];
+    __syncwarp();
+    dft8<float, true>(v);
+}
+
+// R = 2^logW_z whole columns per CTA (at least a warp of them; the surplus
+// lanes of a CTA past Lx work on zeros).  Grid: (nb, Lx / R, Ly).  (A template
+// so that only the translation unit that launches it compiles it.)
+template <int N>
+__global__ void __launch_bounds__(512) k_p3s(MatvecView<float> mv) {
+    static_assert(N == kSplitN, "64-point halves on eight lanes of eight points");
+    if (!grid_begin()) return;
+    const int j = blockIdx.x;                                   // batch slot
+    if (rhs_done(mv, mv.b0 + j)) return;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const Geometry& g = mv.g;
+    const int l = threadIdx.x % kSplitLanes, w = threadIdx.x / kSplitLanes, cols = blockDim.x / kSplitLanes;
+    const int h = l & 1, t = l >> 1;                            // parity, lane of the parity
+    const int ix = blockIdx.y * cols + w, jy = p3_row(blockIdx.z, g.Ly);
+    const bool ok = ix < g.Lx;
+    const int comp = g.Ly * g.Lx * g.Pb;                        // stride between components
+    float2* col = mv.Bxy + j * bxy_elems(g) + (jy * g.Lx + (ok ? ix : 0)) * g.Pb;
+    float2* base = reinterpret_cast<float2*>(smem_raw) + w * kSplitElems;
+    float2 *sm = base + h * kSplitBuf, *sp = base + 2 * kSplitBuf;
+    const int my = jy <= g.Ly / 2 ? jy : g.Ly - jy, fy = jy > g.Ly / 2;
+    const int mx = ix <= g.Lx / 2 ? ix : g.Lx - ix, fx = ix > g.Lx / 2;
+    float2 v[3][8];
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+#pragma unroll
+        for (int m = 0; m < 8; ++m) {
+            const int n = t + 8 * m;
+            v[c][m] = ok && n < g.P ? col[c * comp + n] : make_float2(0.f, 0.f);
+        }
+    // the records of a column, 48 (N/2 + 1) bytes from a 16-byte boundary
+    const float2* line = mv.spec + ((my * g.Hx + (ok ? mx : 0)) * g.Hz) * 6;
+    for (int e = l; e < kSplitSpec / 2; e += kSplitLanes)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(sp + 2 * e)),
+                     "l"(line + 2 * e)
+                     : "memory");
+    asm volatile("cp.async.commit_group;");
+    // w^i, w = W_N^(2 t + h): the powers of two from the table, the others as
+    // products of those
+    float2 wt[8];
+#pragma unroll
+    for (int b = 1; b < 8; b *= 2) {
+        wt[b] = __ldg(mv.tw + (((2 * t + h) * b) % N) * (kTwLen / N));
+#pragma unroll
+        for (int r = 1; r < b; ++r) wt[b + r] = cmul<float>(wt[b], wt[r]);
+    }
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        if (h) {
+#pragma unroll
+            for (int m = 1; m < 8; ++m) v[c][m] = cmul_root<float, false, 16>(v[c][m], m);
+        }
+        split_forward(v[c], sm, t, wt);
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncwarp();
+    // Table 1's sign of the (c, d) component under the mirror flips is
+    // f_c f_d (f = -1 on a mirrored axis): y_c = f_c sum_d G_cd f_d X_d
+    auto flip = [](float2 (&u)[8]) {
+#pragma unroll
+        for (int m = 0; m < 8; ++m) u[m] = cneg<float>(u[m]);
+    };
+    if (fx) flip(v[0]);
+    if (fy) flip(v[1]);
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        const int kz = 2 * (t + 8 * k) + h;
+        const bool fz = k >= 4;                                 // kz > N/2 (at N/2 xz and yz vanish)
+        const float4* r = reinterpret_cast<const float4*>(sp + (fz ? N - kz : kz) * 6);
+        float2 G[6];
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            const float4 f = r[i];
+            G[2 * i] = make_float2(f.x, f.y);
+            G[2 * i + 1] = make_float2(f.z, f.w);
+        }
+        const float2 a = v[0][k], b = v[1][k], d = fz ? cneg<float>(v[2][k]) : v[2][k];
+        v[0][k] = cdot3<float>(G[0], a, G[1], b, G[2], d);
+        v[1][k] = cdot3<float>(G[1], a, G[3], b, G[4], d);
+        const float2 y = cdot3<float>(G[2], a, G[4], b, G[5], d);
+        v[2][k] = fz ? cneg<float>(y) : y;
+    }
+    if (fx) flip(v[0]);
+    if (fy) flip(v[1]);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        split_inverse(v[c], sm, t, wt);
+        // x[t + 8 k] = B_0[k] + W_16^(-k) B_1[k], W_16^(-4) = i: the even lane
+        // of a pair finishes k < 4, the odd one k >= 4
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const float2 lo = v[c][i], hi = v[c][i + 4], s = h ? lo : hi;
+            float2 r;
+            r.x = __shfl_xor_sync(0xffffffffu, s.x, 1);
+            r.y = __shfl_xor_sync(0xffffffffu, s.y, 1);
+            const float2 a = h ? r : lo, b = h ? make_float2(-hi.y, hi.x) : r;
+            const float2 o = i == 0 ? cadd<float>(a, b) : cfma<float>(b, root_v<float, true, 16>(i), a);
+            const int n = t + 8 * (i + 4 * h);
+            if (ok && n < g.P) col[c * comp + n] = o;
+        }
+    }
+}
+
 // ---------------------------------------------------------------- P5
 template <typename T, int N, int LOGW>
 __global__ void __launch_bounds__(kYThreads, sizeof(T) == 4 ? 2 : 1) k_p5(MatvecView<T> mv, const C<IO<T>>* __restrict__ p, C<IO<T>>* __restrict__ y) {
@@ -627,7 +793,12 @@ int launch_p3(const MatvecView<T>& mv, cudaStream_t st) {
     const size_t sm = 3 * (size_t)R * row_ld(N, p3_line_threads(N)) * sizeof(C<T>);
     static std::atomic<size_t> smem_set{0};
     const dim3 grid(mv.nb, (g.Lx + R - 1) / R, g.Ly);
-    if constexpr (Line<N>::ODD) {   // the wide z pass for 3 * 2^a and 5 * 2^a columns
+    if constexpr (split_z<T, N>) {
+        const int cols = split_cols(R);
+        const size_t bytes = (size_t)cols * kSplitElems * sizeof(float2);
+        if (int rc = set_smem((const void*)k_p3s<N>, bytes, smem_set)) return rc;
+        launch_after(k_p3s<N>, dim3(mv.nb, (g.Lx + cols - 1) / cols, g.Ly), cols * kSplitLanes, bytes, st, mv);
+    } else if constexpr (Line<N>::ODD) {   // the wide z pass for 3 * 2^a and 5 * 2^a columns
         if (int rc = set_smem((const void*)k_p3w<T, N>, sm, smem_set)) return rc;
         launch_after(k_p3w<T, N>, grid, R * p3_col_threads(N), sm, st, mv);
     } else {

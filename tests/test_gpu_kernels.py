@@ -150,3 +150,29 @@ def test_tensor_spectrum_pairs(dda, shape):
     # components of a pair are of one size up to the lattice's aspect
     for q in range(6):
         assert err[..., q].max() <= 1e-13 * max(np.abs(half[..., q]).max(), 1e-2 * np.abs(half).max())
+
+
+# ------------------------------------------------- z pass, split columns
+
+# 128-point columns at the ends of their site counts (and the lengths either
+# side, which keep the general kernels), lattices of one x site (fewer columns
+# than a CTA holds) up to several CTAs, tile widths below and above a warp's
+# two columns, a batch
+@pytest.mark.parametrize("P", [48, 49, 57, 64, 65])
+@pytest.mark.parametrize("K,J", [(1, 1), (3, 2), (9, 5)])
+def test_split_columns(dda, P, K, J):
+    case = random_case((K, J, P), seed=P + K, fill=0.8)
+    p = synth.complex_normal(P * K, (2, 3, case.nd), np.complex64)
+    ref = np.stack([odda.direct_matvec(case.coords, case.ainv, case.k, q.astype(np.complex128)) for q in p])
+    with case.lattice() as lat:
+        assert (lat.padded[2] == 128) == (49 <= P <= 64)
+        x = torch.from_numpy(p).to(DEV)
+        got, t0 = [], list(lat.tiles("c64"))
+        for width in ((0, t0[1], t0[1] + 2) if lat.padded[2] == 128 else (t0[1],) * 3):
+            lat.tiles("c64", [t0[0], width, t0[2]])
+            y = torch.empty_like(x)
+            lat.matvec_batch(x, y)
+            got.append(y)
+        assert np.abs(got[0].cpu().numpy() - ref).max() <= 2e-6 * np.abs(ref).max()
+        assert torch.equal(got[0], got[1]) and torch.equal(got[0], got[2])
+
