@@ -34,8 +34,12 @@ void configure_matvec(MatvecView<T>& mv) {
     while (wy > 0 && (1 << (wy - 1)) >= g.K) --wy;          // no wider than the lattice
     // P3: the fewest whole columns per CTA that fill at least two warps
     // exactly (small independent CTAs, many per SM)
+    // (one for FP64: its z pass is bound by the FP64 units, whose share of an
+    // uneven number of CTAs per SM is what small lattices wait for: 82 -> 74 us
+    // at 32^3, the same from 64^3 on)
+    const int least = std::is_same<T, double>::value ? 32 : 64;
     int wz = 0;
-    while (wz < kMaxLogR && (((1 << wz) * tz) < 64 || (((1 << wz) * tz) & 31)) &&
+    while (wz < kMaxLogR && (((1 << wz) * tz) < least || (((1 << wz) * tz) & 31)) &&
            (2 << wz) * tz <= p3_max_threads<T>(g.Lz) && (1 << wz) < g.Lx)
         ++wz;
     // P2/P4: 32 bytes of each column of Bxy per CTA (4 complex64 or 2
