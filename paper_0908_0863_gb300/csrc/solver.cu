@@ -104,16 +104,23 @@ template <int NR>
 __device__ __forceinline__ void final_sums(const double2* __restrict__ part, int nparts, double2 (&out)[NR]) {
     __shared__ double2 sm[NR][kVecThreads];
     __shared__ double2 total[NR];
-    double2 a[NR];
+    // at most kVecBlocks partials: all of a thread's loads go out together
+    constexpr int NU = (kVecBlocks + kVecThreads - 1) / kVecThreads;
+    double2 a[NR], v[NU][NR];
 #pragma unroll
-    for (int r = 0; r < NR; ++r) a[r] = make_double2(0.0, 0.0);
-    for (int i = threadIdx.x; i < nparts; i += kVecThreads)
+    for (int u = 0; u < NU; ++u)
 #pragma unroll
         for (int r = 0; r < NR; ++r) {
-            const double2 v = part[i * kMaxRed + r];
-            a[r].x += v.x;
-            a[r].y += v.y;
+            const int i = threadIdx.x + u * kVecThreads;
+            v[u][r] = i < nparts ? part[i * kMaxRed + r] : make_double2(0.0, 0.0);
         }
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+        a[r] = v[0][r];
+#pragma unroll
+        for (int u = 1; u < NU; ++u)
+            if (threadIdx.x + u * kVecThreads < nparts) { a[r].x += v[u][r].x; a[r].y += v[u][r].y; }
+    }
     block_sums<NR>(a, sm, [&](int r, double2 t) { total[r] = t; });
     __syncthreads();
 #pragma unroll
