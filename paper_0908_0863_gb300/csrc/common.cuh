@@ -111,16 +111,18 @@ bool is_device_ptr(const void* p);
 // predecessors.  grid_begin returns true, from inside the assembly: loads
 // that the compiler takes for invariant (const __restrict__) then sit behind
 // a branch on the wait's result and cannot be moved ahead of it.
-// Two cases keep the ordinary launch.  Grids of more than kAheadThreads
-// threads (about three full waves): early blocks of a kernel keep an SM in
-// the shared-memory split of the kernel before it, and the 256^3 product
-// took 2.93 instead of 2.86 ms with dependent launches throughout, where the
-// one at 64^3 takes 52 instead of 62 us and the one at 16^3 19 instead of
-// 22.5.  And captured streams: the kernels of a replayed graph already start
-// within a microsecond of one another, and with dependent launches among
-// them a solve's iterations took 20% longer (48^3 gradient: 25.2 against
-// 21.3 ms).
-constexpr uint64_t kAheadThreads = 1u << 20;
+// Large grids keep the ordinary launch, more than kAheadThreads threads
+// (about three full waves) or kAheadBlocks blocks (what the SMs hold by
+// count): early blocks of a kernel keep an SM in the shared-memory split of
+// the kernel before it, and each of many short blocks pays for the wait.  The
+// 256^3 product took 2.93 instead of 2.86 ms with dependent launches
+// throughout, and sixteen products of a 6 x 29 x 79 lattice, whose x passes
+// have 61440 blocks, 169 instead of 120 us, where the product at 64^3 takes 52
+// instead of 62 us and the one at 16^3 20 instead of 22.5.  So do captured
+// streams: the kernels of a replayed graph already start within a microsecond
+// of one another, and with dependent launches among them a solve's iterations
+// took 20% longer (48^3 gradient: 25.2 against 21.3 ms).
+constexpr uint64_t kAheadThreads = 1u << 20, kAheadBlocks = 152 * 32;
 __device__ __forceinline__ bool grid_begin() {
     int waited;
     asm volatile("griddepcontrol.launch_dependents;");
@@ -129,7 +131,8 @@ __device__ __forceinline__ bool grid_begin() {
 }
 template <typename... P, typename... A>
 inline cudaError_t launch_after(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
-    bool plain = (uint64_t)grid.x * grid.y * grid.z * block.x > kAheadThreads;
+    const uint64_t blocks = (uint64_t)grid.x * grid.y * grid.z;
+    bool plain = blocks > kAheadBlocks || blocks * block.x > kAheadThreads;
     if (!plain) {
         cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
         const bool asked = cudaStreamIsCapturing(st, &cap) == cudaSuccess;

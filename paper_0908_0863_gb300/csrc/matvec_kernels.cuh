@@ -183,13 +183,14 @@ __global__ void __launch_bounds__(kYThreads) k_p1(MatvecView<T> mv, const C<IO<T
 // more), and the row side whole 32-byte sectors of Wz rows.  A CTA holds
 // rows_groups(N, Wz, c128) tiles of consecutive z, each with its own region of
 // shared memory: more than one for the wide mappings, whose few threads per
-// line would otherwise make CTAs of a warp or less, and for 8-byte reals on
-// short rows, where a CTA of half a warp takes the FP64 units as long as a
-// full one (64-point rows of complex128 at 32^3: 28 -> 19 us a pass).
+// line would otherwise make CTAs of a warp or less, and on short rows, to
+// fill a warp (complex64) or two (8-byte reals, where half a warp takes the
+// FP64 units as long as a full one: 64-point rows of complex128 at 32^3 28 ->
+// 19 us a pass).
 // Forward (P2): Ay rows -> transform -> Bxy.  Inverse (P4): Bxy ->
 // transform -> the first K outputs into Ay.  Grid: (z tiles, Ly, 3 nb).
 __host__ __device__ constexpr int rows_groups(int N, int Wz, bool c128) {
-    const int threads = Wz * map_threads(N, c128), want = map_wide(N, c128) ? 128 : c128 ? 64 : 1;
+    const int threads = Wz * map_threads(N, c128), want = map_wide(N, c128) ? 128 : c128 ? 64 : 32;
     return threads < want ? want / threads : 1;
 }
 
