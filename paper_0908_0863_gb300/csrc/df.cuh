@@ -31,6 +31,9 @@ struct DF {
     __host__ __device__ __forceinline__ DF(float h, float l) : hi(h), lo(l) {}
 };
 
+// Scalar operations: the reference form of the steps, checked on the host
+// against exact arithmetic; the kernels run their paired forms below.
+//
 // The high product, rounded on its own: the device compiler never contracts
 // __fmul_rn into the sum that follows it, which would count the product's
 // rounding error twice.
@@ -69,7 +72,6 @@ __host__ __device__ __forceinline__ DF operator*(DF a, DF b) {
 __host__ __device__ __forceinline__ DF fma(DF a, DF b, DF c) { return a * b + c; }
 __host__ __device__ __forceinline__ float fma(float a, float b, float c) { return ::fmaf(a, b, c); }
 __host__ __device__ __forceinline__ double fma(double a, double b, double c) { return ::fma(a, b, c); }
-__host__ __device__ __forceinline__ double to_double(DF a) { return (double)a.hi + (double)a.lo; }
 
 // Complex double-float, 16 bytes: the high parts of (re, im), then the low
 // parts.  On the device both parts go through the arithmetic as one pair, on
