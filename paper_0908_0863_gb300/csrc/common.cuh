@@ -100,45 +100,27 @@ bool is_device_ptr(const void* p);
         if (e__ != cudaSuccess) return ::dda::cuda_fail(e__, what);      \
     } while (0)
 
-// Dependent launches: a kernel launched with launch_after may be scheduled
-// while the kernel before it in the stream still runs or drains, so that its
-// launch latency and its start overlap that kernel's end.  Such a kernel
-// calls grid_begin in every thread before it touches memory that an earlier
-// kernel writes or reads: it lets the next kernel of the stream be scheduled
-// in turn, then waits until all earlier kernels have completed and their
-// writes are visible.  (Both are no-ops after an ordinary launch.)  A kernel
-// must not return without that wait: its completion stands for that of its
-// predecessors.  grid_begin returns true, from inside the assembly: loads
-// that the compiler takes for invariant (const __restrict__) then sit behind
-// a branch on the wait's result and cannot be moved ahead of it.
-// Large grids keep the ordinary launch, more than kAheadThreads threads
-// (about three full waves) or kAheadBlocks blocks (what the SMs hold by
-// count): early blocks of a kernel keep an SM in the shared-memory split of
-// the kernel before it, and each of many short blocks pays for the wait.  The
-// 256^3 product took 2.93 instead of 2.86 ms with dependent launches
-// throughout, and sixteen products of a 6 x 29 x 79 lattice, whose x passes
-// have 61440 blocks, 169 instead of 120 us, where the product at 64^3 takes 52
-// instead of 62 us and the one at 16^3 20 instead of 22.5.  So do captured
-// streams: the kernels of a replayed graph already start within a microsecond
-// of one another, and with dependent launches among them a solve's iterations
-// took 20% longer (48^3 gradient: 25.2 against 21.3 ms).
-constexpr uint64_t kAheadThreads = 1u << 20, kAheadBlocks = 152 * 32;
-__device__ __forceinline__ bool grid_begin() {
-    int waited;
+// Dependent launches: a kernel launched with launch_after(ahead = true) may be
+// scheduled while the kernel before it in the stream still runs or drains, so
+// that its launch latency and its start overlap that kernel's end.  Such a
+// kernel calls grid_begin in every thread before it touches memory that an
+// earlier kernel writes or reads: it lets the next kernel of the stream be
+// scheduled in turn, then waits until all earlier kernels have completed and
+// their writes are visible.  It must not return without that wait: its
+// completion stands for that of its predecessors.  The wait orders ordinary
+// loads and stores; read-only loads (__ldg, const __restrict__ parameters)
+// assume memory that nothing writes while the kernel is resident, which starts
+// before the wait.  So what earlier kernels write (vectors, work arrays, status
+// words) is read with ordinary loads, and only a context's tables, bit fields,
+// ranks and spectrum, complete before its first product, with read-only ones.
+__device__ __forceinline__ void grid_begin(int ahead) {
+    if (!ahead) return;   // (also in an ordinary launch every block would pay for the wait)
     asm volatile("griddepcontrol.launch_dependents;");
-    asm volatile("griddepcontrol.wait;\n\tmov.u32 %0, 1;" : "=r"(waited) : : "memory");
-    return waited != 0;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 template <typename... P, typename... A>
-inline cudaError_t launch_after(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
-    const uint64_t blocks = (uint64_t)grid.x * grid.y * grid.z;
-    bool plain = blocks > kAheadBlocks || blocks * block.x > kAheadThreads;
-    if (!plain) {
-        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-        const bool asked = cudaStreamIsCapturing(st, &cap) == cudaSuccess;
-        if (!asked) cudaGetLastError();
-        plain = !asked || cap != cudaStreamCaptureStatusNone;
-    }
+inline cudaError_t launch_after(bool ahead, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                                A&&... args) {
     cudaLaunchAttribute at{};
     at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at.val.programmaticStreamSerializationAllowed = 1;
@@ -148,7 +130,7 @@ inline cudaError_t launch_after(void (*kernel)(P...), dim3 grid, dim3 block, siz
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cfg.attrs = &at;
-    cfg.numAttrs = plain ? 0 : 1;
+    cfg.numAttrs = ahead ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
 

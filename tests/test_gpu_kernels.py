@@ -95,6 +95,47 @@ def test_products_in_stream_order(dda, shape, side):
             assert torch.equal(a, b)
 
 
+# products that read the previous product's output with nothing between them,
+# in all three arithmetics, against the same sequence replayed from a captured
+# graph, where every pass is an ordinary launch.  (64, 64, 48) is just below
+# the block limit of dependent launches in the complex64 x passes (4608 of
+# 4864) and (64, 64, 52) just above it, with the other passes below; a batch
+# of five takes the 16-byte arithmetics through several chunks, each one's last
+# pass followed by the first of the next
+@pytest.mark.parametrize("shape,nb", [((6, 5, 4), 1), ((6, 5, 4), 5), ((40, 24, 33), 1), ((40, 24, 33), 3),
+                                      ((64, 64, 48), 1), ((64, 64, 52), 1), ((17, 60, 49), 5)])
+@pytest.mark.parametrize("dtype", ["c64", "c128", "c128df"])
+def test_dependent_products_equal_captured(dda, shape, nb, dtype):
+    case = random_case(shape, seed=nb, fill=0.8)
+    real = np.complex64 if dtype == "c64" else np.complex128
+    kind = "c128df" if dtype == "c128df" else None
+    with case.lattice() as lat:
+        p = torch.from_numpy(synth.complex_normal(6, (nb, 3, case.nd), real)).to(DEV)
+        a, b = torch.empty_like(p), torch.empty_like(p)
+
+        def chain():
+            dda.dda_matvec_batch(lat.ctx, p, a, dtype=kind)
+            for _ in range(3):
+                dda.dda_matvec_batch(lat.ctx, a, b, dtype=kind)
+                dda.dda_matvec_batch(lat.ctx, b, a, dtype=kind)
+
+        chain()   # the workspace grows here, not under capture
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            chain()
+        graph.replay()
+        torch.cuda.synchronize()
+        want = a.clone(), b.clone()
+        assert torch.isfinite(torch.view_as_real(want[0])).all()
+        for _ in range(4):
+            a.zero_()
+            b.zero_()
+            chain()
+            torch.cuda.synchronize()
+            assert torch.equal(a, want[0]) and torch.equal(b, want[1])
+
+
 # ------------------------------------------------------------ double-float
 
 # vectors around the ends of the range that is split and widened on the
