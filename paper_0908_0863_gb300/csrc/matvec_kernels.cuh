@@ -187,7 +187,9 @@ __global__ void __launch_bounds__(kYThreads) k_p1(MatvecView<T> mv, const C<IO<T
 // line would otherwise make CTAs of a warp or less, and on short rows, to
 // fill a warp (complex64) or two (8-byte reals, where half a warp takes the
 // FP64 units as long as a full one: 64-point rows of complex128 at 32^3 28 ->
-// 19 us a pass).
+// 19 us a pass).  A lattice with fewer tiles than that along z has a CTA of
+// those alone: surplus threads would transform zeros (complex128 41 x 90 x 2:
+// 69 -> 22.5 us a pass; 6 x 15 x 1, sixteen at a time: 14.5 -> 10.4).
 // Forward (P2): Ay rows -> transform -> Bxy.  Inverse (P4): Bxy ->
 // transform -> the first K outputs into Ay.  Grid: (z tiles, Ly, 3 nb).
 __host__ __device__ constexpr int rows_groups(int N, int Wz, bool c128) {
@@ -783,15 +785,16 @@ template <typename T, bool INV, int N, int LOGZ>
 int launch_rows_w(const MatvecView<T>& mv, cudaStream_t st) {
     const Geometry& g = mv.g;
     constexpr bool c128 = sizeof(T) == 8;
-    constexpr int Wz = 1 << LOGZ, G = rows_groups(N, Wz, c128), threads = G * Wz * Map<T, N>::T_;
-    if constexpr (threads > rows_max_threads(N, c128)) {
+    constexpr int Wz = 1 << LOGZ, G = rows_groups(N, Wz, c128), tile = Wz * Map<T, N>::T_;
+    if constexpr (G * tile > rows_max_threads(N, c128)) {
         return fail(DDA_ERR_ARG, "x pass tile wider than a CTA");
     } else {
-        const size_t sm = rows_smem_elems(N, Wz, c128) * sizeof(C<T>);
+        const int tiles = (g.P + Wz - 1) / Wz, groups = std::min(G, tiles);
+        const size_t sm = (size_t)groups * rows_tile_elems(N, Wz, c128) * sizeof(C<T>);
         static std::atomic<size_t> smem_set{0};
         if (int rc = set_smem((const void*)k_rows<T, INV, N, LOGZ>, sm, smem_set)) return rc;
-        const dim3 grid((unsigned)((g.P + G * Wz - 1) / (G * Wz)), g.Ly, 3 * mv.nb);
-        launch_pass(mv, k_rows<T, INV, N, LOGZ>, grid, threads, sm, st);
+        const dim3 grid((unsigned)((tiles + G - 1) / G), g.Ly, 3 * mv.nb);
+        launch_pass(mv, k_rows<T, INV, N, LOGZ>, grid, groups * tile, sm, st);
         DDA_LAUNCH_CHECK(INV ? "P4 x-inverse" : "P2 x-forward");
         return 0;
     }

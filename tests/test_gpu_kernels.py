@@ -171,6 +171,23 @@ def test_short_rows(dda, K, P):
             assert np.abs(y.cpu().numpy() - ref).max() <= tol * np.abs(ref).max()
 
 
+# fewer z tiles than a CTA of the x passes holds (it then has those alone), as
+# many, and one more, in batches
+@pytest.mark.parametrize("K", [2, 6, 14, 50])
+@pytest.mark.parametrize("P", [1, 2, 5, 8, 9, 33])
+@pytest.mark.parametrize("dtype", ["c64", "c128", "c128df"])
+def test_few_z_tiles(dda, K, P, dtype):
+    case = random_case((K, 5, P), seed=K * P, fill=0.9)
+    p = synth.complex_normal(K + P, (3, 3, case.nd), np.complex64 if dtype == "c64" else np.complex128)
+    ref = np.stack([odda.direct_matvec(case.coords, case.ainv, case.k, q.astype(np.complex128)) for q in p])
+    with case.lattice() as lat:
+        x = torch.from_numpy(p).to(DEV)
+        y = torch.empty_like(x)
+        dda.dda_matvec_batch(lat.ctx, x, y, dtype="c128df" if dtype == "c128df" else None)
+    tol = {"c64": 2e-6, "c128": 1e-13, "c128df": 1e-12}[dtype]
+    assert np.abs(y.cpu().numpy() - ref).max() <= tol * np.abs(ref).max()
+
+
 # --------------------------------------------------------- tensor spectrum
 
 # paired even and odd lines on every axis, lines of one site among them
