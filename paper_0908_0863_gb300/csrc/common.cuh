@@ -101,22 +101,29 @@ bool is_device_ptr(const void* p);
     } while (0)
 
 // Dependent launches: a kernel launched with launch_after(ahead = true) may be
-// scheduled while the kernel before it in the stream still runs or drains, so
-// that its launch latency and its start overlap that kernel's end.  Such a
-// kernel calls grid_begin in every thread before it touches memory that an
-// earlier kernel writes or reads: it lets the next kernel of the stream be
-// scheduled in turn, then waits until all earlier kernels have completed and
-// their writes are visible.  It must not return without that wait: its
-// completion stands for that of its predecessors.  The wait orders ordinary
-// loads and stores; read-only loads (__ldg, const __restrict__ parameters)
-// assume memory that nothing writes while the kernel is resident, which starts
-// before the wait.  So what earlier kernels write (vectors, work arrays, status
-// words) is read with ordinary loads, and only a context's tables, bit fields,
-// ranks and spectrum, complete before its first product, with read-only ones.
-__device__ __forceinline__ void grid_begin(int ahead) {
-    if (!ahead) return;   // (also in an ordinary launch every block would pay for the wait)
-    asm volatile("griddepcontrol.launch_dependents;");
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+// scheduled as soon as the blocks of the kernel before it in the stream have
+// ended, so that its launch overlaps the completion of that kernel.  Such a
+// kernel calls grid_wait in every thread before it touches memory that an
+// earlier kernel writes or reads: it waits until all earlier kernels have
+// completed and their writes are visible.  It must not return without that
+// wait: its completion stands for that of its predecessors.  The wait orders
+// ordinary loads and stores; read-only loads (__ldg, const __restrict__
+// parameters) assume memory that nothing writes while the kernel is resident,
+// which may start before the wait ends.  So what earlier kernels write
+// (vectors, work arrays, status words) is read with ordinary loads, and only a
+// context's tables, bit fields, ranks and spectrum, complete before its first
+// product, with read-only ones.
+// No kernel lets its successor start earlier than that
+// (griddepcontrol.launch_dependents).  Called at the start, several later
+// kernels pile up on the SMs that have room and their blocks are spread
+// unevenly (complex64 24 x 40 x 40 took 40 us that way, 34 with ordinary
+// launches, 20.7 this way; complex128 32^3 203 us that way, 138 with ordinary
+// launches).  Called before the final stores, it changed the compiler's
+// schedule of them (x pass of 192-point rows, four of 95 x 94 x 105: 102 -> 122
+// us).  In an ordinary launch the wait is skipped: with many short blocks it
+// alone made passes up to 1.9 times as long.
+__device__ __forceinline__ void grid_wait(int ahead) {
+    if (ahead) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 template <typename... P, typename... A>
 inline cudaError_t launch_after(bool ahead, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,

@@ -72,17 +72,9 @@ static int launch_chunk(const MatvecView<T>& mv, const C<IO<T>>* p, C<IO<T>>* y,
 }
 
 // Whether the passes of a product on this stream may be dependent launches
-// (common.cuh): complex64 ones outside captured streams.  With 8-byte reals
-// the waiting blocks hold back the pass they wait for, whose few blocks share
-// the FP64 units: limited to 2^16 threads, complex128 products took up to
-// twice as long (14 x 21 x 16, four at a time: 0.51 of the speed) and 0.92 of
-// the speed on average over 133, double-float ones down to 0.71.  The kernels of a
-// replayed graph already start within a microsecond of one another, and with
-// dependent launches among them a solve's iterations took 20% longer (48^3
-// gradient: 25.2 against 21.3 ms).
-template <typename T>
+// (common.cuh): not in captured streams, where the kernels of a replayed graph
+// already start within a microsecond of one another
 static bool may_run_ahead(cudaStream_t st) {
-    if (!std::is_same<T, float>::value) return false;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) {
         cudaGetLastError();
@@ -94,7 +86,7 @@ static bool may_run_ahead(cudaStream_t st) {
 template <typename T>
 int launch_matvec(const MatvecView<T>& mv, const C<IO<T>>* p, C<IO<T>>* y, cudaStream_t st) {
     if (mv.nb < 1 || mv.slots < 1) return fail(DDA_ERR_ARG, "matvec: empty batch");
-    const int ahead = may_run_ahead<T>(st);
+    const int ahead = may_run_ahead(st);
     for (int b0 = 0; b0 < mv.nb; b0 += mv.slots) {
         MatvecView<T> m = mv;
         m.b0 = b0;

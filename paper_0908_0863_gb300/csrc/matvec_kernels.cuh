@@ -105,10 +105,10 @@ __host__ __device__ __forceinline__ int64_t bxy_elems(const Geometry& g) { retur
 // ---------------------------------------------------------------- P1
 template <typename T, int N, int LOGW>
 __global__ void __launch_bounds__(kYThreads) k_p1(MatvecView<T> mv, const C<IO<T>>* p) {
-    // (p may be an earlier kernel's output: no __restrict__, see grid_begin)
+    // (p may be an earlier kernel's output: no __restrict__, see grid_wait)
     // the three components of a site share its occupancy and rank lookup:
     // each thread gathers all three and transforms them as three lines
-    grid_begin(mv.ahead);
+    grid_wait(mv.ahead);
     const int j = blockIdx.z;                                  // batch slot
     const int b = mv.b0 + j;
     if (rhs_done(mv, b)) return;
@@ -206,7 +206,7 @@ __host__ __device__ constexpr int rows_tile_elems(int N, int Wz, bool c128) {
 
 template <typename T, bool INV, int N, int LOGZ>
 __global__ void __launch_bounds__(rows_max_threads(N, sizeof(T) == 8)) k_rows(MatvecView<T> mv) {
-    grid_begin(mv.ahead);
+    grid_wait(mv.ahead);
     const int c = blockIdx.z % 3, j = blockIdx.z / 3;      // component, batch slot
     if (rhs_done(mv, mv.b0 + j)) return;
     extern __shared__ unsigned char smem_raw[];
@@ -332,7 +332,7 @@ __device__ __forceinline__ void put_line(C<T> (&v)[3][8], int c, const C<T> (&u)
 // DFTs, and the store of k < P.  Grid: (nb, Lx / R, Ly).
 template <typename T, int N>
 __global__ void __launch_bounds__(p3_max_threads<T>(N)) k_p3(MatvecView<T> mv) {
-    grid_begin(mv.ahead);
+    grid_wait(mv.ahead);
     const int j = blockIdx.x;                                   // batch slot
     if (rhs_done(mv, mv.b0 + j)) return;
     extern __shared__ unsigned char smem_raw[];
@@ -417,7 +417,7 @@ __global__ void __launch_bounds__(p3_max_threads<T>(N)) k_p3(MatvecView<T> mv) {
 template <typename T, int N>
 __global__ void __launch_bounds__(p3_max_threads<T>(N)) __maxnreg__(sizeof(T) == 4 ? 128 : 255) k_p3w(MatvecView<T> mv) {
     static_assert(Line<N>::ODD, "k_p3w takes 3 * 2^a and 5 * 2^a columns (their spectrum lines are [6][Hz])");
-    grid_begin(mv.ahead);
+    grid_wait(mv.ahead);
     const int j = blockIdx.x;                                   // batch slot
     if (rhs_done(mv, mv.b0 + j)) return;
     extern __shared__ unsigned char smem_raw[];
@@ -563,7 +563,7 @@ __device__ __forceinline__ void split_inverse(float2 (&v)[8], float2* __restrict
 template <int N>
 __global__ void __launch_bounds__(512) k_p3s(MatvecView<float> mv) {
     static_assert(N == kSplitN, "64-point halves on eight lanes of eight points");
-    grid_begin(mv.ahead);
+    grid_wait(mv.ahead);
     const int j = blockIdx.x;                                   // batch slot
     if (rhs_done(mv, mv.b0 + j)) return;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -662,8 +662,8 @@ __global__ void __launch_bounds__(512) k_p3s(MatvecView<float> mv) {
 // ---------------------------------------------------------------- P5
 template <typename T, int N, int LOGW>
 __global__ void __launch_bounds__(kYThreads, sizeof(T) == 4 ? 2 : 1) k_p5(MatvecView<T> mv, const C<IO<T>>* p, C<IO<T>>* __restrict__ y) {
-    // (p may be an earlier kernel's output: no __restrict__, see grid_begin)
-    grid_begin(mv.ahead);
+    // (p may be an earlier kernel's output: no __restrict__, see grid_wait)
+    grid_wait(mv.ahead);
     const int c = blockIdx.z % 3, j = blockIdx.z / 3;      // component, batch slot
     const int b = mv.b0 + j;
     if (rhs_done(mv, b)) return;
@@ -746,16 +746,14 @@ inline int set_smem(const void* fn, size_t bytes, std::atomic<size_t>& done) {
 
 // ------------------------------------------------- per-length launchers
 // Launches a pass, as a dependent launch where the product allows it
-// (mv.ahead, complex64) and the grid is small: beyond kAheadThreads threads or
-// kAheadBlocks blocks (what the SMs hold by count) the overlap of two launches
-// is a small part of a pass, early blocks keep an SM in the shared-memory split
-// of the kernel before, and every block pays for the wait.  Measured on 261
-// complex64 products (log-uniform edges up to 300, batches of 1, 4 and 16) at
-// limits of 2^14 to 2^19 threads: 1.11 times as fast as ordinary launches on
-// average at 2^14, 1.15 at 2^16, 1.17 at 2^19, where 211 are more than 3%
-// faster (16^3 22.6 -> 17.2 us, 64^3 59.5 -> 49.0) and three more than 3% slower (at worst
-// 28.3 -> 30.4 us).
-constexpr uint64_t kAheadThreads = 1u << 19, kAheadBlocks = 152 * 32;
+// (mv.ahead) and the grid is small: up to kAheadThreads threads (about three
+// full waves) and kAheadBlocks blocks (what the SMs hold by count); beyond that
+// the overlap is a small part of a pass, and each of many short blocks would
+// pay for the wait.  Against ordinary launches, on products of log-uniform edges
+// up to 300 in batches of 1, 4 and 16: complex64 1.15 times as fast on average
+// (324 products; 16^3 22.6 -> 18.2 us, 64^3 61.1 -> 48.4), complex128 1.15
+// (188), double-float 1.24 (201), and one of them all slower by more than 3%.
+constexpr uint64_t kAheadThreads = 1u << 20, kAheadBlocks = 152 * 32;
 template <typename T, typename... P, typename... A>
 inline void launch_pass(const MatvecView<T>& mv, void (*kernel)(MatvecView<T>, P...), dim3 grid, unsigned threads,
                         size_t smem, cudaStream_t st, A&&... args) {
