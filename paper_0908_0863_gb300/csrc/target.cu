@@ -151,14 +151,22 @@ __global__ void k_site_ranks(TargetView tv, int64_t n, uint32_t* __restrict__ ou
 // E = e exp(i k khat . r) = [e exp(i k (khat_y j + khat_z k))] exp(i k khat_x i):
 // one phase per row (j, k) and one per x index, so that a site costs three
 // complex products instead of a sine and cosine (FP64 arithmetic bounds this
-// kernel: at 200^3, 4.19 M sites, it took 424 us with a sincos per site,
-// 126 us this way; writing the field alone takes 30 us at the measured copy
-// rate).  A CTA takes the rows b, b + G, ...
-// (interleaved: a target's first and last planes are often nearly empty),
-// kIncRows at a time.
+// kernel: at 200^3, 4.19 M sites, it took 424 us with a sincos per site, 125 us
+// this way; writing the field alone takes 30 us at the measured copy rate).
+// The angles carry their rounding errors, so that the field is within 1.1e-16
+// of the exact one however long the lattice is (rounded angles: 2.6e-15 at
+// 200^3).  A CTA takes the rows b, b + G, ... (interleaved: a target's first and
+// last planes are often nearly empty), kIncRows at a time, and shares their
+// sites out evenly over its threads, however long a row is (5 x 200 x 200 14 us;
+// with a warp per row, whose lanes are idle past a row's end, 39, with a sincos
+// per site 23).  With one site along x a row is a line along y instead, or each
+// site would need a row's phase (1 x 512 x 512 23 us, that way 39, with a sincos
+// per site 27).
 constexpr int kIncThreads = 512;
-constexpr int kIncRows = 128;
+constexpr int kIncRows = 512;
 constexpr int kIncUnroll = 4;
+__host__ __device__ __forceinline__ bool inc_along_y(const Geometry& g) { return g.K == 1; }
+__host__ __device__ __forceinline__ int inc_len(const Geometry& g) { return inc_along_y(g) ? g.J : g.K; }
 
 // one axis of the wave vector as an unevaluated sum of two doubles, and the
 // phase n of that axis added to an angle held the same way
@@ -182,40 +190,44 @@ __global__ void __launch_bounds__(kIncThreads) k_incident(TargetView tv, Geometr
                                                           double2* __restrict__ E) {
     __shared__ double2 px[kMaxEdge];
     __shared__ double2 F[kIncRows][3];
-    const int nrows = g.J * g.P, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int i = threadIdx.x; i < g.K; i += kIncThreads) px[i] = phase(angle_at(ax, i));
+    const bool along_y = inc_along_y(g);
+    const int len = inc_len(g), nrows = (int)(g.nsites / len);
+    for (int i = kIncThreads - 1 - threadIdx.x; i < len; i += kIncThreads)   // (the last threads first: the first have a row)
+        px[i] = phase(angle_at(along_y ? ay : ax, i));
     for (int base = blockIdx.x; base < nrows; base += kIncRows * gridDim.x) {
         const int left = (nrows - base + gridDim.x - 1) / gridDim.x, cnt = left < kIncRows ? left : kIncRows;
-        __syncthreads();
         if (threadIdx.x < cnt) {
             const int row = base + threadIdx.x * gridDim.x;
-            const double2 f = phase(angle_add(angle_at(ay, row % g.J), angle_at(az, row / g.J)));
+            const double2 f = phase(along_y ? angle_at(az, row) : angle_add(angle_at(ay, row % g.J), angle_at(az, row / g.J)));
             F[threadIdx.x][0] = cmul<double>(e0, f);
             F[threadIdx.x][1] = cmul<double>(e1, f);
             F[threadIdx.x][2] = cmul<double>(e2, f);
         }
         __syncthreads();
-        for (int q = warp; q < cnt; q += kIncThreads / 32) {
-            const int s0 = (base + q * gridDim.x) * g.K;
-            for (int i0 = lane; i0 < g.K; i0 += 32 * kIncUnroll) {
-                uint32_t word[kIncUnroll], rank[kIncUnroll];
+        // the sites of these rows, end to end: number t is site t % len of row t / len
+        const uint32_t sites = (uint32_t)cnt * len;
+        for (uint32_t t0 = threadIdx.x; t0 < sites; t0 += kIncThreads * kIncUnroll) {
+            uint32_t word[kIncUnroll], rank[kIncUnroll], bit[kIncUnroll], q[kIncUnroll], i[kIncUnroll];
 #pragma unroll
-                for (int u = 0; u < kIncUnroll; ++u) {
-                    const int i = i0 + 32 * u;
-                    word[u] = i < g.K ? __ldg(tv.occ + ((s0 + i) >> 5)) : 0u;
-                    rank[u] = i < g.K ? __ldg(tv.rank + ((s0 + i) >> 5)) : 0u;
-                }
+            for (int u = 0; u < kIncUnroll; ++u) {
+                const uint32_t t = t0 + u * kIncThreads;
+                q[u] = t / (uint32_t)len;
+                i[u] = t - q[u] * len;
+                const uint32_t s = (base + q[u] * gridDim.x) * len + i[u];
+                bit[u] = s & 31;
+                word[u] = t < sites ? __ldg(tv.occ + (s >> 5)) : 0u;
+                rank[u] = t < sites ? __ldg(tv.rank + (s >> 5)) : 0u;
+            }
 #pragma unroll
-                for (int u = 0; u < kIncUnroll; ++u) {
-                    const int i = i0 + 32 * u, bit = (s0 + i) & 31;
-                    if (!((word[u] >> bit) & 1u)) continue;
-                    const int64_t r = rank[u] + __popc(word[u] & ((1u << bit) - 1u));
-                    const double2 x = px[i];
+            for (int u = 0; u < kIncUnroll; ++u) {
+                if (!((word[u] >> bit[u]) & 1u)) continue;
+                const int64_t r = rank[u] + __popc(word[u] & ((1u << bit[u]) - 1u));
+                const double2 x = px[i[u]];
 #pragma unroll
-                    for (int c = 0; c < 3; ++c) E[c * g.nd + r] = cmul<double>(F[q][c], x);
-                }
+                for (int c = 0; c < 3; ++c) E[c * g.nd + r] = cmul<double>(F[q[u]][c], x);
             }
         }
+        __syncthreads();   // F is written again
     }
 }
 
@@ -480,8 +492,8 @@ int launch_incident(const TargetView& tv, const Geometry& g, double k, const dou
         a[i].hi = k * khat[i];
         a[i].lo = std::fma(k, khat[i], -a[i].hi);
     }
-    // at least a row per warp, at most two CTAs per SM (each one computes the K phases of the x axis)
-    const int rows = g.J * g.P, per = kIncThreads / 32;
+    // a site per thread, whole rows, at most two CTAs per SM (each one computes the phases along a row)
+    const int len = inc_len(g), rows = (int)(g.nsites / len), per = (kIncThreads + len - 1) / len;
     const unsigned grid = (unsigned)std::min(152 * 2, (rows + per - 1) / per);
     k_incident<<<grid, kIncThreads, 0, st>>>(tv, g, a[0], a[1], a[2], make_double2(e0[0], e0[1]),
                                              make_double2(e0[2], e0[3]), make_double2(e0[4], e0[5]), E);

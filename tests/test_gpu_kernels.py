@@ -25,10 +25,12 @@ def dda():
 
 # ------------------------------------------------ incident field, cross sections
 
-# rows of 1 to 512 sites (the unrolled x loop takes 128 at a time), and
-# 40,000 rows (more than one CTA round of 128 rows x 304 CTAs)
+# rows of 1 to 512 sites (lattices of one x site take their rows along y), fewer
+# and more sites than a CTA's threads, and 40,000 and 160,000 rows (the latter
+# more than one round of 512 rows x 304 CTAs)
 @pytest.mark.parametrize("shape,fill", [((1, 1, 1), 1.0), ((129, 3, 2), 0.5), ((512, 2, 3), 0.3), ((33, 17, 5), 0.6),
-                                        ((3, 200, 200), 0.4)])
+                                        ((3, 200, 200), 0.4), ((1, 400, 400), 0.3), ((2, 400, 400), 0.1),
+                                        ((512, 1, 9), 0.8)])
 def test_incident_field_edges(dda, shape, fill):
     case = random_case(shape, seed=sum(shape), fill=fill, two_materials=False)
     kh = synth.random_direction(7)[0]
