@@ -378,7 +378,8 @@ int dda_solve_batch(dda_ctx* ctx, int nb, const void* einc, void* p, int method,
  *   C_abs = 4 pi k sum_j sum_c [-Im(alpha^-1_jc) - (2/3) k^3] |P_jc|^2
  *   C_sca = C_ext - C_abs.
  * einc, p: host or device [3][N_d] complex128; out: host double[3] =
- * {C_ext, C_abs, C_sca}.  FP64 reductions in a fixed order (deterministic).
+ * {C_ext, C_abs, C_sca}.  FP64 reductions in a fixed order (deterministic, and
+ * the same alone as at any place of a batch).
  * Synchronises the stream.
  */
 int dda_cross_sections(dda_ctx* ctx, const void* einc, const void* p, double* out, void* stream);

@@ -515,7 +515,7 @@ int dda_init_lattice(dda_ctx** out, const int32_t shape[3], const uint32_t* occu
         probe.take<cdf>(3 * (size_t)n_materials);
         probe.take<cdf>(nspec);
         probe.take<cdf>(kTwEntries);
-        probe.take<double2>(xsec_scratch_elems());
+        probe.take<double2>(xsec_scratch_elems(g));
         probe.take<double2>(material_sums_scratch_elems(g));
         probe.take<int>(4);
         a0.cap = probe.used + 256;
@@ -540,7 +540,7 @@ int dda_init_lattice(dda_ctx** out, const int32_t shape[3], const uint32_t* occu
     c->jac_df = a0.take<cdf>(3 * (size_t)n_materials);
     c->spec_df = a0.take<cdf>(nspec);
     c->tw_df = a0.take<cdf>(kTwEntries);
-    c->xsec = a0.take<double2>(xsec_scratch_elems());
+    c->xsec = a0.take<double2>(xsec_scratch_elems(g));
     c->msum = a0.take<double2>(material_sums_scratch_elems(g));
     int* flags = a0.take<int>(4);
     c->bytes_fixed = (int64_t)a0.cap;

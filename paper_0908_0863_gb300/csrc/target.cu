@@ -242,7 +242,15 @@ __global__ void __launch_bounds__(kIncThreads) k_incident(TargetView tv, Geometr
 // right-hand side (its two vectors take 59 us at the measured copy rate).
 constexpr int kRedThreads = 256;
 constexpr int kRedBlocks = 1024;
-constexpr int kRedUnroll = 4;
+constexpr int kRedUnroll = 2;   // dipoles in flight per thread, all three components each
+
+// blocks of one right-hand side's sums over n dipoles or sites, `each` or more
+// per thread.  They follow from the lattice alone, so that the sums are added
+// in the same order alone and at any place of a batch.
+inline int red_blocks(int64_t n, int each) {
+    const int64_t per = (int64_t)kRedThreads * each;
+    return (int)std::max<int64_t>(1, std::min<int64_t>(kRedBlocks, (n + per - 1) / per));
+}
 
 // sums of a and b over the block, valid in thread 0
 __device__ __forceinline__ double2 block_sum2(double a, double b) {
@@ -276,25 +284,29 @@ __global__ void __launch_bounds__(kRedThreads) k_xsec_partial(TargetView tv, Geo
     const int stride = gridDim.x * kRedThreads, first = blockIdx.x * kRedThreads + threadIdx.x;
     if (ONE) {
         const int nd = (int)g.nd;
-        for (int c = 0; c < 3; ++c) {
-            const double2 *Ec = E + c * g.nd, *Pc = P + c * g.nd;
-            double sq = 0.0;
-            for (int i = first; i < nd; i += kRedUnroll * stride) {
-                double2 e[kRedUnroll], p[kRedUnroll];
+        double sq[3] = {0.0, 0.0, 0.0};
+        for (int i = first; i < nd; i += kRedUnroll * stride) {
+            double2 e[kRedUnroll][3], p[kRedUnroll][3];
 #pragma unroll
-                for (int u = 0; u < kRedUnroll; ++u) {
+            for (int u = 0; u < kRedUnroll; ++u)
+#pragma unroll
+                for (int c = 0; c < 3; ++c) {
                     const int n = i + u * stride;
-                    e[u] = n < nd ? Ec[n] : make_double2(0.0, 0.0);
-                    p[u] = n < nd ? Pc[n] : make_double2(0.0, 0.0);
+                    e[u][c] = n < nd ? E[c * g.nd + n] : make_double2(0.0, 0.0);
+                    p[u][c] = n < nd ? P[c * g.nd + n] : make_double2(0.0, 0.0);
                 }
 #pragma unroll
-                for (int u = 0; u < kRedUnroll; ++u) {
-                    ext = fma(e[u].x, p[u].y, fma(-e[u].y, p[u].x, ext));   // Im(conj(e) p)
-                    sq = fma(p[u].x, p[u].x, fma(p[u].y, p[u].y, sq));
+            for (int u = 0; u < kRedUnroll; ++u) {
+                if (i + u * stride >= nd) break;
+#pragma unroll
+                for (int c = 0; c < 3; ++c) {
+                    ext = fma(e[u][c].x, p[u][c].y, fma(-e[u][c].y, p[u][c].x, ext));   // Im(conj(e) p)
+                    sq[c] = fma(p[u][c].x, p[u][c].x, fma(p[u][c].y, p[u][c].y, sq[c]));
                 }
             }
-            abs_ += weight[c] * sq;
         }
+#pragma unroll
+        for (int c = 0; c < 3; ++c) abs_ += weight[c] * sq[c];
     } else {
         const int n = (int)g.nsites;
         for (int s = first; s < n; s += stride) {
@@ -501,31 +513,29 @@ int launch_incident(const TargetView& tv, const Geometry& g, double k, const dou
     return 0;
 }
 
-size_t xsec_scratch_elems() { return kRedBlocks + kXsecBatch; }
+size_t xsec_scratch_elems(const Geometry& g) { return kXsecBatch * (size_t)(1 + red_blocks(g.nsites, 1)); }
 
 int launch_cross_sections(const TargetView& tv, const Geometry& g, double k, const double2* ainv, int nb,
                           const double2* E, const double2* P, double2* scratch, cudaStream_t st) {
     const bool one = g.nmat == 1;
-    const int64_t need = ((one ? g.nd : g.nsites) + kRedThreads - 1) / kRedThreads;
-    const unsigned blocks = (unsigned)std::max<int64_t>(1, std::min<int64_t>(kRedBlocks / nb, need));
+    const int blocks = one ? red_blocks(g.nd, kRedUnroll) : red_blocks(g.nsites, 1);
     const size_t sm = 3 * (size_t)g.nmat * sizeof(double);
     const dim3 grid(blocks, nb);
     double2* part = scratch + kXsecBatch;
     if (one) k_xsec_partial<true><<<grid, kRedThreads, sm, st>>>(tv, g, k * k * k, ainv, E, P, part);
     else k_xsec_partial<false><<<grid, kRedThreads, sm, st>>>(tv, g, k * k * k, ainv, E, P, part);
     DDA_LAUNCH_CHECK("cross-section partial sums");
-    k_xsec_final<<<nb, kRedThreads, 0, st>>>(part, (int)blocks, scratch);
+    k_xsec_final<<<nb, kRedThreads, 0, st>>>(part, blocks, scratch);
     DDA_LAUNCH_CHECK("cross-section final sum");
     return 0;
 }
 
 int launch_csca(const TargetView& tv, const Geometry& g, double k, const double2* ainv, const double2* P,
                 const double2* AP, const double2* AhP, double2* scratch, cudaStream_t st) {
-    const unsigned blocks =
-        (unsigned)std::min<int64_t>(kRedBlocks, std::max<int64_t>(1, (g.nsites + kRedThreads - 1) / kRedThreads));
+    const int blocks = red_blocks(g.nsites, 1);
     k_csca_partial<<<blocks, kRedThreads, 0, st>>>(tv, g, k * k * k, ainv, P, AP, AhP, scratch + kXsecBatch);
     DDA_LAUNCH_CHECK("C_sca partial sums");
-    k_xsec_final<<<1, kRedThreads, 0, st>>>(scratch + kXsecBatch, (int)blocks, scratch);
+    k_xsec_final<<<1, kRedThreads, 0, st>>>(scratch + kXsecBatch, blocks, scratch);
     DDA_LAUNCH_CHECK("C_sca final sum");
     return 0;
 }

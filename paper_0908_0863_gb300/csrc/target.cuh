@@ -33,7 +33,8 @@ int launch_incident(const TargetView& tv, const Geometry& g, double k, const dou
 
 // right-hand sides of one launch_cross_sections call (at most)
 constexpr int kXsecBatch = 32;
-size_t xsec_scratch_elems();
+// elements of their scratch
+size_t xsec_scratch_elems(const Geometry& g);
 // scratch[b] receives {sum Im(E_b^* P_b), sum [-Im ainv - 2/3 k^3] |P_b|^2} for b < nb <= kXsecBatch
 // (E, P: [nb][3][N_d])
 int launch_cross_sections(const TargetView& tv, const Geometry& g, double k, const double2* ainv, int nb,

@@ -64,6 +64,20 @@ def test_cross_sections_batches(dda, nb, two):
         assert got[b, 2] == got[b, 0] - got[b, 1]
 
 
+# a right-hand side's sums are added in one order, alone or at any place of a
+# batch (21,600 dipoles or 24,000 sites: 43 and 94 blocks a right-hand side)
+@pytest.mark.parametrize("two", [False, True])
+@pytest.mark.parametrize("nb", [2, 32, 33, 40])
+def test_cross_sections_do_not_depend_on_the_batch(dda, nb, two):
+    case = random_case((40, 30, 20), seed=nb, fill=0.9, two_materials=two)
+    E = torch.from_numpy(synth.complex_normal(nb, (nb, 3, case.nd))).to(DEV)
+    P = (0.2 - 0.1j) * E + 0.05 * torch.from_numpy(synth.complex_normal(nb + 1, (nb, 3, case.nd))).to(DEV)
+    with case.lattice() as lat:
+        got = lat.cross_sections_batch(E, P)
+        for b in range(nb):
+            assert np.array_equal(got[b], lat.cross_sections(E[b], P[b])), b
+
+
 # ------------------------------------------------------ dependent launches
 
 # products queued back to back with other work of the same stream between
