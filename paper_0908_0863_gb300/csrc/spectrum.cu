@@ -13,14 +13,12 @@
 // 1/(Lx Ly Lz) (the iDFT normalisation of Sec. 3 step 4) and copied to
 // complex64 and double-float form for the mixed-precision matvec.
 //
-// A mirrored line is even or odd (Table 1), and so is its transform.  An
-// even line a and an odd one b of two components therefore share one
-// transform: with X the DFT of a + b, the DFT of a is (X[k] + X[L-k]) / 2 and
-// that of b (X[k] - X[L-k]) / 2.  On each axis two components are odd and
-// four even, so the six take four transforms (this step is bound by the FP64
-// units).  The halvings are left to the final scale: with the yz component
-// doubled at the start, the two components of every pair carry the same power
-// of two, so that neither adds more than its share to the other's rounding.
+// Every component is transformed by itself.  (A mirrored line is even or odd,
+// and so is its transform, so that an even and an odd component could share
+// one DFT: four transforms for six lines, which saves about 0.7 of the 6.5 ms of
+// a 100^3 context.  But then the larger line's rounding goes into the smaller
+// one too: the xy component's error at 9 x 33 x 65 grew from 4.0e-16 to 7.7e-16
+// of its norm, the whole spectrum's at 100^3 from 4.9e-16 to 5.1e-16.)
 #include "fft.cuh"
 #include "matvec.cuh"
 #include "spectrum.cuh"
@@ -29,24 +27,14 @@ namespace dda {
 
 namespace {
 
-// Components transformed together on an axis: job q takes the even component
-// pair_even and, where there is one, the odd component pair_odd (else -1)
-__device__ __forceinline__ int pair_even(int axis, int q) {
-    constexpr int e[3][4] = {{0, 3, 4, 5}, {0, 2, 3, 5}, {0, 1, 3, 5}};
-    return e[axis][q];
-}
-__device__ __forceinline__ int pair_odd(int axis, int q) {
-    constexpr int o[3][4] = {{1, 2, -1, -1}, {1, 4, -1, -1}, {2, 4, -1, -1}};
-    return o[axis][q];
-}
-// power of two a component carries through the pairings (the yz component's
-// starting 2 included), as its reciprocal
-__device__ __forceinline__ double pair_unscale(int m) {
-    constexpr double u[6] = {0.125, 0.125, 0.125, 0.5, 0.125, 1.0};
-    return u[m];
+// Table 1, row = axis (x, y, z), column = component
+__device__ __forceinline__ double table1_sign(int axis, int m) {
+    // sign -1 when the component pairs the mirrored axis with another axis
+    const int a[6] = {0, 0, 0, 1, 1, 2}, b[6] = {0, 1, 2, 1, 2, 2};
+    return ((a[m] == axis) != (b[m] == axis)) ? -1.0 : 1.0;
 }
 
-// t_m at r = (i, j, k) != 0 (the yz component doubled):
+// t_m at r = (i, j, k) != 0:
 //   exp(ikr)/r^3 [ k^2 (r_a r_b - r^2 d_ab) + (ikr - 1)/r^2 (3 r_a r_b - r^2 d_ab) ]
 __global__ void k_section1(Geometry g, double kw, double2* __restrict__ t1) {
     const int64_t n = g.nsites;
@@ -76,46 +64,33 @@ __global__ void k_section1(Geometry g, double kw, double2* __restrict__ t1) {
                 out[m] = make_double2(e.x * inner.x - e.y * inner.y, e.x * inner.y + e.y * inner.x);
             }
         }
-        out[4].x *= 2.0;
-        out[4].y *= 2.0;
         for (int m = 0; m < 6; ++m) t1[m * n + s] = out[m];
     }
 }
 
 constexpr int kV = 8;
 
-// point n of a mirrored line, or of a pair of them: src(i) is entry i < nline
-// of the even line, src2(i) of the odd one
-template <typename Src, typename Src2>
-__device__ __forceinline__ double2 mirrored(int n, int nline, int N, bool pair, Src src, Src2 src2) {
-    if (n < nline) {
-        double2 v = src(n);
-        if (pair) { const double2 o = src2(n); v.x += o.x; v.y += o.y; }
-        return v;
-    }
-    if (n > N - nline) {
-        double2 v = src(N - n);
-        if (pair) { const double2 o = src2(N - n); v.x -= o.x; v.y -= o.y; }
-        return v;
-    }
-    return make_double2(0.0, 0.0);
-}
-
-// x lines: rows of K values (t1 [6][P][J][K]) -> rows of Hx ([6][P][J][Hx]); grid (row tiles, 4 jobs)
+// x lines: rows of K values (t1 [6][P][J][K]) -> rows of Hx ([6][P][J][Hx])
 __global__ void __launch_bounds__(512) k_tensor_x(Geometry g, int logW, const double2* __restrict__ tw,
                                                   const double2* __restrict__ in, double2* __restrict__ out) {
     extern __shared__ unsigned char smem_raw[];
     double2* buf = reinterpret_cast<double2*>(smem_raw);
     const int W = 1 << logW, ld = W + 1, N = g.Lx;
-    const int64_t rows = (int64_t)g.P * g.J, r0 = (int64_t)blockIdx.x * W;
-    const int me = pair_even(0, blockIdx.y), mo = pair_odd(0, blockIdx.y);
+    const int64_t rows_per_m = (int64_t)g.P * g.J, nrows = 6 * rows_per_m;
+    const int64_t r0 = (int64_t)blockIdx.x * W;
     for (int e = threadIdx.x; e < W * N; e += blockDim.x) {
         const int w = e / N, n = e - w * N;
         const int64_t row = r0 + w;
         double2 v = make_double2(0.0, 0.0);
-        if (row < rows) {
-            const double2 *a = in + (me * rows + row) * g.K, *b = in + (mo * rows + row) * g.K;
-            v = mirrored(n, g.K, N, mo >= 0, [&](int i) { return a[i]; }, [&](int i) { return b[i]; });
+        if (row < nrows) {
+            const int m = (int)(row / rows_per_m);
+            if (n < g.K) {
+                v = in[row * g.K + n];
+            } else if (n > N - g.K) {
+                v = in[row * g.K + (N - n)];
+                const double sg = table1_sign(0, m);
+                v.x *= sg; v.y *= sg;
+            }
         }
         buf[n * ld + w] = v;
     }
@@ -124,24 +99,15 @@ __global__ void __launch_bounds__(512) k_tensor_x(Geometry g, int logW, const do
     for (int e = threadIdx.x; e < W * g.Hx; e += blockDim.x) {
         const int w = e / g.Hx, n = e - w * g.Hx;
         const int64_t row = r0 + w;
-        if (row >= rows) continue;
-        const double2 x = buf[n * ld + w];
-        double2* oe = out + (me * rows + row) * g.Hx + n;
-        if (mo < 0) {
-            *oe = x;
-        } else {
-            const double2 y = buf[(n ? N - n : 0) * ld + w];
-            *oe = make_double2(x.x + y.x, x.y + y.y);
-            out[(mo * rows + row) * g.Hx + n] = make_double2(x.x - y.x, x.y - y.y);
-        }
+        if (row < nrows) out[row * g.Hx + n] = buf[n * ld + w];
     }
 }
 
 // strided lines along y (axis 1) or z (axis 2) on arrays whose rows are Hx
 // long.  in: [6][n_outer][n_line][Hx] slices -> out: [6][n_outer][H][Hx]
 // (y pass: outer = P, line = J -> Hy; z pass: the line is the outermost
-// index of [6][P][Hy][Hx] -> the z-line layout of spec_index, scaled, with
-// the complex64 and double-float copies).  Grid (x tiles, outer, 4 jobs).
+// index of [6][P][Hy][Hx] -> the z-line layout of spec_index, with the
+// complex64 and double-float copies).
 template <int AXIS>
 __global__ void __launch_bounds__(512) k_tensor_col(Geometry g, int logW, const double2* __restrict__ tw,
                                                     const double2* __restrict__ in, double2* __restrict__ out,
@@ -154,49 +120,51 @@ __global__ void __launch_bounds__(512) k_tensor_col(Geometry g, int logW, const 
     const int H = AXIS == 1 ? g.Hy : g.Hz;
     const int x0 = blockIdx.x * W;
     const int outer = blockIdx.y;   // y pass: z plane k; z pass: row my
-    const int me = pair_even(AXIS, blockIdx.z), mo = pair_odd(AXIS, blockIdx.z);
-    // first element of component m's line at x = 0, and the step along it
-    auto in_base = [&](int m) -> int64_t {
-        return AXIS == 1 ? (((int64_t)m * g.P + outer) * g.J) * g.Hx : ((int64_t)m * g.P * g.Hy + outer) * g.Hx;
-    };
-    const int64_t in_step = AXIS == 1 ? g.Hx : (int64_t)g.Hy * g.Hx;
-    const double2 *a = in + in_base(me), *b = in + in_base(mo >= 0 ? mo : me);
+    const int m = blockIdx.z;
+    // element (line point n, column x) of the input and output
+    int64_t in_base, in_step, out_base, out_step;
+    if (AXIS == 1) {
+        in_base = (((int64_t)m * g.P + outer) * g.J) * g.Hx;
+        in_step = g.Hx;
+        out_base = (((int64_t)m * g.P + outer) * g.Hy) * g.Hx;
+        out_step = g.Hx;
+    } else {
+        in_base = ((int64_t)m * g.P * g.Hy + outer) * g.Hx;
+        in_step = (int64_t)g.Hy * g.Hx;
+        out_base = ((int64_t)m * g.Hz * g.Hy + outer) * g.Hx;
+        out_step = (int64_t)g.Hy * g.Hx;
+    }
+    const double sg = table1_sign(AXIS, m);
     for (int e = threadIdx.x; e < W * N; e += blockDim.x) {
         const int n = e >> logW, w = e & (W - 1), x = x0 + w;
         double2 v = make_double2(0.0, 0.0);
-        if (x < g.Hx)
-            v = mirrored(n, nline, N, mo >= 0, [&](int i) { return a[i * in_step + x]; },
-                         [&](int i) { return b[i * in_step + x]; });
+        if (x < g.Hx) {
+            if (n < nline) {
+                v = in[in_base + n * in_step + x];
+            } else if (n > N - nline) {
+                v = in[in_base + (N - n) * in_step + x];
+                v.x *= sg; v.y *= sg;
+            }
+        }
         buf[n * ld + w] = v;
     }
     __syncthreads();
     fft_tile<double, kV, false>(buf, ld, logW, N, tw);
-    auto store = [&](int m, int n, int x, double2 v) {
+    for (int e = threadIdx.x; e < W * H; e += blockDim.x) {
+        const int n = e >> logW, w = e & (W - 1), x = x0 + w;
+        if (x >= g.Hx) continue;
+        double2 v = buf[n * ld + w];
+        v.x *= scale; v.y *= scale;
         if (AXIS == 1) {
-            out[(((int64_t)m * g.P + outer) * g.Hy + n) * g.Hx + x] = v;
+            out[out_base + n * out_step + x] = v;
         } else {
             // final spectrum: every z line contiguous (spec_index), so the z
             // pass reads a column's line in one stream
-            const double f = scale * pair_unscale(m);
-            v.x *= f;
-            v.y *= f;
             const int64_t o = spec_index(g, outer, x, n, m);
             out[o] = v;
             const cdf d = from_io<DF>(v);
             outdf[o] = d;
             out32[o] = d.h;   // the nearest floats
-        }
-    };
-    for (int e = threadIdx.x; e < W * H; e += blockDim.x) {
-        const int n = e >> logW, w = e & (W - 1), x = x0 + w;
-        if (x >= g.Hx) continue;
-        const double2 p = buf[n * ld + w];
-        if (mo < 0) {
-            store(me, n, x, p);
-        } else {
-            const double2 q = buf[(n ? N - n : 0) * ld + w];
-            store(me, n, x, make_double2(p.x + q.x, p.y + q.y));
-            store(mo, n, x, make_double2(p.x - q.x, p.y - q.y));
         }
     }
 }
@@ -246,8 +214,8 @@ int build_spectrum(const Geometry& g, double k, const double2* tw, double2* s0, 
         const int logW = pick_logW_rows(g.Lx), W = 1 << logW;
         const size_t sm = (size_t)g.Lx * (W + 1) * sizeof(double2);
         if ((rc = smem_attr((const void*)k_tensor_x, sm))) return rc;
-        const int64_t rows = (int64_t)g.P * g.J;
-        k_tensor_x<<<dim3((unsigned)((rows + W - 1) / W), 4), W * g.Lx / kV, sm, st>>>(g, logW, tw, s0, s1);
+        const int64_t rows = 6ll * g.P * g.J;
+        k_tensor_x<<<(unsigned)((rows + W - 1) / W), W * g.Lx / kV, sm, st>>>(g, logW, tw, s0, s1);
         DDA_LAUNCH_CHECK("tensor x DFT");
     }
     // y lines
@@ -255,7 +223,7 @@ int build_spectrum(const Geometry& g, double k, const double2* tw, double2* s0, 
         const int logW = pick_logW_cols(g.Ly, g.Hx), W = 1 << logW;
         const size_t sm = (size_t)g.Ly * (W + 1) * sizeof(double2);
         if ((rc = smem_attr((const void*)k_tensor_col<1>, sm))) return rc;
-        dim3 grid((g.Hx + W - 1) / W, g.P, 4);
+        dim3 grid((g.Hx + W - 1) / W, g.P, 6);
         k_tensor_col<1><<<grid, W * g.Ly / kV, sm, st>>>(g, logW, tw, s1, s0, 1.0, nullptr, nullptr);
         DDA_LAUNCH_CHECK("tensor y DFT");
     }
@@ -264,7 +232,7 @@ int build_spectrum(const Geometry& g, double k, const double2* tw, double2* s0, 
         const int logW = pick_logW_cols(g.Lz, g.Hx), W = 1 << logW;
         const size_t sm = (size_t)g.Lz * (W + 1) * sizeof(double2);
         if ((rc = smem_attr((const void*)k_tensor_col<2>, sm))) return rc;
-        dim3 grid((g.Hx + W - 1) / W, g.Hy, 4);
+        dim3 grid((g.Hx + W - 1) / W, g.Hy, 6);
         const double scale = 1.0 / ((double)g.Lx * g.Ly * g.Lz);
         k_tensor_col<2><<<grid, W * g.Lz / kV, sm, st>>>(g, logW, tw, s0, spec64, scale, spec32, specdf);
         DDA_LAUNCH_CHECK("tensor z DFT");
