@@ -299,7 +299,7 @@ __device__ __forceinline__ void dft3(C<T>& a, C<T>& b, C<T>& c) {
     const T h = (T)0.86602540378443864676;   // sqrt(3) / 2
     const C<T> s = cadd<T>(b, c), d = csub<T>(b, c);
     C<T> m;
-    if constexpr (std::is_same<T, DF>::value) m = csub<DF>(a, cdf{__fmul2_rn(s.h, both(0.5f)), __fmul2_rn(s.l, both(0.5f))});
+    if constexpr (std::is_same<T, DF>::value) m = csub<DF>(a, cdf{mul2(s.h, both(0.5f)), mul2(s.l, both(0.5f))});
     else m = mk<T>(a.x - (T)0.5 * s.x, a.y - (T)0.5 * s.y);
     const C<T> r = cscale<T>(rot90<T, INV>(d), h);
     a = cadd<T>(a, s);
@@ -588,8 +588,8 @@ __device__ __forceinline__ C<T> cmul_root(C<T> x, int e) {
             const cdf p = cr > 0 ? x : cneg<DF>(x), q = sr > 0 ? rot90<DF, true>(x) : rot90<DF, false>(x);
             return cscale<DF>(cadd<DF>(p, q), h);
         } else {
-        const T c = (T)(cr > 0 ? 1.0 : -1.0), s = (T)(sr > 0 ? 1.0 : -1.0);
-        return mk<T>((c * x.x - s * x.y) * h, (c * x.y + s * x.x) * h);
+            const T c = (T)(cr > 0 ? 1.0 : -1.0), s = (T)(sr > 0 ? 1.0 : -1.0);
+            return mk<T>((c * x.x - s * x.y) * h, (c * x.y + s * x.x) * h);
         }
     }
     return cmul<T>(x, root_v<T, INV, V>(e));
