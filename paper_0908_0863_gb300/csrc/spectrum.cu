@@ -18,7 +18,9 @@
 // one DFT: four transforms for six lines, which saves about 0.7 of the 6.5 ms of
 // a 100^3 context.  But then the larger line's rounding goes into the smaller
 // one too: the xy component's error at 9 x 33 x 65 grew from 4.0e-16 to 7.7e-16
-// of its norm, the whole spectrum's at 100^3 from 4.9e-16 to 5.1e-16.)
+// of its norm, the whole spectrum's at 100^3 from 4.9e-16 to 5.1e-16.)  The
+// double-float copy is a kernel of its own: written by the z pass, whose rows
+// are short scattered pieces, it made a 100^3 context take 6.50 instead of 6.45 ms.
 #include "fft.cuh"
 #include "matvec.cuh"
 #include "spectrum.cuh"
@@ -96,22 +98,21 @@ __global__ void __launch_bounds__(512) k_tensor_x(Geometry g, int logW, const do
     }
     __syncthreads();
     fft_tile<double, kV, false>(buf, ld, logW, N, tw);
-    for (int e = threadIdx.x; e < W * g.Hx; e += blockDim.x) {
-        const int w = e / g.Hx, n = e - w * g.Hx;
+    for (int e = threadIdx.x; e < W * N; e += blockDim.x) {
+        const int w = e / N, n = e - w * N;
         const int64_t row = r0 + w;
-        if (row < nrows) out[row * g.Hx + n] = buf[n * ld + w];
+        if (row < nrows && n < g.Hx) out[row * g.Hx + n] = buf[n * ld + w];
     }
 }
 
 // strided lines along y (axis 1) or z (axis 2) on arrays whose rows are Hx
 // long.  in: [6][n_outer][n_line][Hx] slices -> out: [6][n_outer][H][Hx]
 // (y pass: outer = P, line = J -> Hy; z pass: the line is the outermost
-// index of [6][P][Hy][Hx] -> the z-line layout of spec_index, with the
-// complex64 and double-float copies).
+// index of [6][P][Hy][Hx] -> the z-line layout of spec_index).
 template <int AXIS>
 __global__ void __launch_bounds__(512) k_tensor_col(Geometry g, int logW, const double2* __restrict__ tw,
                                                     const double2* __restrict__ in, double2* __restrict__ out,
-                                                    double scale, float2* __restrict__ out32, cdf* __restrict__ outdf) {
+                                                    double scale, float2* __restrict__ out32) {
     extern __shared__ unsigned char smem_raw[];
     double2* buf = reinterpret_cast<double2*>(smem_raw);
     const int W = 1 << logW, ld = W + 1;
@@ -162,11 +163,15 @@ __global__ void __launch_bounds__(512) k_tensor_col(Geometry g, int logW, const 
             // pass reads a column's line in one stream
             const int64_t o = spec_index(g, outer, x, n, m);
             out[o] = v;
-            const cdf d = from_io<DF>(v);
-            outdf[o] = d;
-            out32[o] = d.h;   // the nearest floats
+            if (out32) out32[o] = make_float2((float)v.x, (float)v.y);
         }
     }
+}
+
+// the double-float copy of n spectrum entries
+__global__ void __launch_bounds__(256) k_spec_to_df(const double2* __restrict__ in, cdf* __restrict__ out, int64_t n) {
+    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x)
+        out[e] = from_io<DF>(in[e]);
 }
 
 int pick_logW_rows(int N) {   // rows of length N, V = 8 values per thread, <= 512 threads
@@ -224,18 +229,23 @@ int build_spectrum(const Geometry& g, double k, const double2* tw, double2* s0, 
         const size_t sm = (size_t)g.Ly * (W + 1) * sizeof(double2);
         if ((rc = smem_attr((const void*)k_tensor_col<1>, sm))) return rc;
         dim3 grid((g.Hx + W - 1) / W, g.P, 6);
-        k_tensor_col<1><<<grid, W * g.Ly / kV, sm, st>>>(g, logW, tw, s1, s0, 1.0, nullptr, nullptr);
+        k_tensor_col<1><<<grid, W * g.Ly / kV, sm, st>>>(g, logW, tw, s1, s0, 1.0, nullptr);
         DDA_LAUNCH_CHECK("tensor y DFT");
     }
-    // z lines, scaled, with the complex64 and double-float copies
+    // z lines, scaled, with the complex64 copy
     {
         const int logW = pick_logW_cols(g.Lz, g.Hx), W = 1 << logW;
         const size_t sm = (size_t)g.Lz * (W + 1) * sizeof(double2);
         if ((rc = smem_attr((const void*)k_tensor_col<2>, sm))) return rc;
         dim3 grid((g.Hx + W - 1) / W, g.Hy, 6);
         const double scale = 1.0 / ((double)g.Lx * g.Ly * g.Lz);
-        k_tensor_col<2><<<grid, W * g.Lz / kV, sm, st>>>(g, logW, tw, s0, spec64, scale, spec32, specdf);
+        k_tensor_col<2><<<grid, W * g.Lz / kV, sm, st>>>(g, logW, tw, s0, spec64, scale, spec32);
         DDA_LAUNCH_CHECK("tensor z DFT");
+    }
+    {
+        const size_t n = 6ull * g.Hz * g.Hy * g.Hx;
+        k_spec_to_df<<<(unsigned)std::min<size_t>((n + 255) / 256, 152 * 16), 256, 0, st>>>(spec64, specdf, (int64_t)n);
+        DDA_LAUNCH_CHECK("spectrum double-float copy");
     }
     return 0;
 }
