@@ -238,8 +238,9 @@ __global__ void __launch_bounds__(kIncThreads) k_incident(TargetView tv, Geometr
 // the weight is a constant of the component, so the compressed vectors are
 // streamed without a look at the bit field and a value costs four FP64
 // operations; with more, each occupied site looks its materials up and takes
-// the weights from shared memory.  At 200^3 and one material 222 -> 95 us a
-// right-hand side (its two vectors take 59 us at the measured copy rate).
+// the weights from shared memory.  At 200^3 222 -> 101 us a right-hand side
+// with one material, 171 us with two (its two vectors take 59 us at the
+// measured copy rate).
 constexpr int kRedThreads = 256;
 constexpr int kRedBlocks = 1024;
 constexpr int kRedUnroll = 2;   // dipoles in flight per thread, all three components each
